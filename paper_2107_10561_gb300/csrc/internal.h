@@ -231,6 +231,17 @@ struct Level {
   uint32_t* mt16 = nullptr;       // [N][32] the smoothing step's residual block as packed BF16 (lo << 16 | hi)
 };
 
+// Work space of the dense products and inverses of kernels_dense.cu: digit operands, one block, pivots.
+struct DenseWork {
+  static constexpr int kSlots = 6;
+  void* dig[kSlots] = {};
+  int* exps[kSlots] = {};
+  long long halves[kSlots] = {}, nexp[kSlots] = {};
+  double* tmp = nullptr;
+  int *piv = nullptr, *from = nullptr;
+  long long ntmp = 0, npiv = 0, nfrom = 0;
+};
+
 struct Hierarchy {
   stm_params p{};
   std::vector<Level> L;
@@ -250,6 +261,10 @@ struct Hierarchy {
   long long *cs_off = nullptr, *cs_pos = nullptr;
   int *cs_rowslab = nullptr, *cs_perm = nullptr;
   double *cs_store = nullptr, *cs_u = nullptr, *cs_v = nullptr, *cs_mu = nullptr, *cs_mv = nullptr;
+  DenseWork dw[2];                // coarse factorisation: one work space per elimination chain
+  double* cs_raw = nullptr;       // dense blocks of J_0 in slab order
+  cudaStream_t chain_stream = nullptr;  // the second chain's stream
+  cudaEvent_t chain_ev[2] = {};
   int* dflag = nullptr;           // device flags: [0] singular flag, [1..2] bad cell (int64 split)
   int* dkerr = nullptr;           // device error word of the tensor-core pipelines (bounded waits)
   long long* dbad = nullptr;
@@ -316,6 +331,34 @@ stm_status assemble_level(Hierarchy& H, int g, double nu, cudaStream_t s);
 stm_status factor_level(Hierarchy& H, int g, cudaStream_t s);
 stm_status factor_coarse(Hierarchy& H, cudaStream_t s);
 stm_status ensure_transpose(Hierarchy& H, int g, cudaStream_t s);
+// Dense FP64 products and inverses on the tensor cores (kernels_dense.cu). An operand is cut into digits in
+// a slot of the work space: as row operand (the left factor, scaled per row) or as column operand.
+struct DenseSlice {
+  int slot = 0;
+  bool column = false;
+  const double* src = nullptr;  // rows x cols, row-major
+  long long ld = 0;
+  int rows = 0, cols = 0;
+};
+// C = [C0 +] alpha A B (m x k times k x n); trans: C^T is stored; columns [skip0, skip1) of C are left alone
+struct DenseProduct {
+  int a = 0, b = 0;  // slots
+  int m = 0, n = 0, k = 0;
+  double alpha = 1.0;
+  const double* C0 = nullptr;
+  long long ldc0 = 0;
+  double* C = nullptr;
+  long long ldc = 0;
+  int trans = 0, skip0 = 0, skip1 = 0;
+};
+stm_status dense_reserve(DenseWork& w, int slot, long long rows, long long cols);
+stm_status dense_reserve_inverse(DenseWork& w, long long n);  // slots 0 and 1, the block, the pivots
+void dense_free(DenseWork& w);
+// flag: device word set to 1 when an entry is not finite (slices) or a pivot is zero or not finite (inverse)
+stm_status dense_slice(DenseWork& w, const DenseSlice* sl, int count, int* flag, cudaStream_t s);      // <= 6
+stm_status dense_products(const DenseWork& w, const DenseProduct* pr, int count, cudaStream_t s);      // <= 4
+stm_status dense_inverse(DenseWork& w, double* A, int n, double* out, int* flag, cudaStream_t s);      // A is overwritten
+long long dense_max_inverse();
 
 // y = alpha*A x + beta_y*y (+ b): mode 0: y = A x; 1: y = b - A x; 2: y += A x
 stm_status csr_apply(const long long* rowptr, const int* col, const double* val, long long nrows, long long nnz,

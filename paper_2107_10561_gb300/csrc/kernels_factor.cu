@@ -278,64 +278,6 @@ __global__ void k_gj_colswap(double* A, long long n, int k, const int* piv) {
 // (X_b = Z_b - W_b X_{b+1}), and finally the slab permutation is undone.
 // ---------------------------------------------------------------------------------------------
 
-// C = beta C + alpha A B, row-major, FP64. 64x64 tile per 256-thread CTA, 4x4 outputs per thread.
-__global__ void __launch_bounds__(256) k_dgemm_rm(int m, int n, int k, double alpha, const double* __restrict__ A,
-                                                  long long lda, const double* __restrict__ B, long long ldb,
-                                                  double beta, double* __restrict__ C, long long ldc) {
-  __shared__ double As[16][64 + 1];
-  __shared__ double Bs[16][64];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
-  double acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-  for (int k0 = 0; k0 < k; k0 += 16) {
-    for (int e = threadIdx.x; e < 64 * 16; e += 256) {
-      const int rr = e / 16, kk = e - rr * 16;
-      const int gr = r0 + rr, gk = k0 + kk;
-      As[kk][rr] = (gr < m && gk < k) ? A[(long long)gr * lda + gk] : 0.0;
-      const int kb = e / 64, cc = e - kb * 64;
-      const int gkb = k0 + kb, gc = c0 + cc;
-      Bs[kb][cc] = (gkb < k && gc < n) ? B[(long long)gkb * ldb + gc] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        a[q] = As[kk][ty + 16 * q];
-        b[q] = Bs[kk][tx + 16 * q];
-      }
-#pragma unroll
-      for (int qa = 0; qa < 4; ++qa)
-#pragma unroll
-        for (int qb = 0; qb < 4; ++qb) acc[qa][qb] += a[qa] * b[qb];
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int qa = 0; qa < 4; ++qa)
-#pragma unroll
-    for (int qb = 0; qb < 4; ++qb) {
-      const int gr = r0 + ty + 16 * qa, gc = c0 + tx + 16 * qb;
-      if (gr < m && gc < n) {
-        double* c = C + (long long)gr * ldc + gc;
-        *c = (beta == 0.0 ? 0.0 : beta * *c) + alpha * acc[qa][qb];
-      }
-    }
-}
-
-static void dgemm(int m, int n, int k, double alpha, const double* A, long long lda, const double* B, long long ldb,
-                  double beta, double* C, long long ldc, cudaStream_t s) {
-  if (m <= 0 || n <= 0) return;
-  dim3 grid((n + 63) / 64, (m + 63) / 64);
-  k_dgemm_rm<<<grid, 256, 0, s>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
-  note_launch();
-}
-
 // Dense slab blocks from the CSR of J_0: row r of slab b (permuted index pr = iperm[r]) scatters its
 // entries into D_b (same slab), Lo_b (slab b-1) or Up_b (slab b+1); anything else flags an error.
 __global__ void k_slab_blocks(const long long* __restrict__ rowptr, const int* __restrict__ col,
@@ -364,23 +306,8 @@ __global__ void k_slab_blocks(const long long* __restrict__ rowptr, const int* _
   }
 }
 
-// Single-CTA Gauss-Jordan inverse of a small dense block (in place, through shared memory).
-__global__ void __launch_bounds__(1024) k_block_inverse_smem(double* __restrict__ M, int n, int* flag) {
-  extern __shared__ double sm[];
-  double* A = sm;
-  short* perm = reinterpret_cast<short*>(A + (size_t)n * n);
-  __shared__ int s_piv, s_bad;
-  if (threadIdx.x == 0) s_bad = 0;
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) A[e] = M[e];
-  __syncthreads();
-  if (!gj_invert_smem(A, perm, n, &s_piv, &s_bad)) {
-    if (threadIdx.x == 0) atomicExch(flag, 1);
-    return;
-  }
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) M[e] = A[e];
-}
-
-// Explicit inverse of a dense n x n block in global memory, one pivot at a time (larger blocks).
+// Explicit inverse of a dense n x n block in global memory, one pivot at a time (blocks with more rows
+// than a cluster's shared memory holds as one panel, see dense_max_inverse).
 static void block_inverse_global(double* M, long long n, int* piv, double* scal, int* flag, cudaStream_t s) {
   const int vb = (int)std::min<long long>((n + 255) / 256, sm_count() * 8LL);
   const int mb = (int)std::min<long long>((n * n + 255) / 256, sm_count() * 32LL);
@@ -468,17 +395,13 @@ static void coarse_slabs(const Level& L, int tw, std::vector<int>& iperm, std::v
   }
 }
 
-// In-place inverse of one dense FP64 block (Gauss-Jordan, partial pivoting): in shared memory when it
-// fits, else column by column in global memory.
-static void invert_block(double* Db, long long nb, int* piv, double* scal, int* flag, int maxsm, cudaStream_t s) {
-  const size_t smem = sizeof(double) * nb * nb + sizeof(short) * nb + 16;
-  if (smem + 64 <= (size_t)maxsm) {
-    cudaFuncSetAttribute(k_block_inverse_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_block_inverse_smem<<<1, 1024, smem, s>>>(Db, (int)nb, flag);
-    note_launch();
-  } else {
-    block_inverse_global(Db, nb, piv, scal, flag, s);
-  }
+// Inverse of one dense FP64 block (Gauss-Jordan, partial pivoting); M is overwritten.
+static stm_status invert_block(DenseWork& w, double* M, long long nb, double* out, int* flag, double* scal,
+                               cudaStream_t s) {
+  if (nb <= dense_max_inverse()) return dense_inverse(w, M, (int)nb, out, flag, s);
+  block_inverse_global(M, nb, w.piv, scal, flag, s);
+  STM_CUDA(cudaMemcpyAsync(out, M, sizeof(double) * nb * nb, cudaMemcpyDeviceToDevice, s));
+  return STM_OK;
 }
 
 // Twisted block factorisation of J_0 in slab order, eliminated from both ends towards slab t = nx / 2
@@ -497,15 +420,14 @@ static void invert_block(double* Db, long long nb, int* piv, double* scal, int* 
 static stm_status twisted_slab_factors(Hierarchy& H, const Level& L, const std::vector<long long>& off,
                                        const std::vector<int>& iperm, const std::vector<int>& blk, double* raw,
                                        const std::vector<long long>& dpos, const std::vector<long long>& lpos,
-                                       const std::vector<long long>& upos, int* piv, double* scal, int maxsm,
-                                       cudaStream_t s) {
+                                       const std::vector<long long>& upos, double* scal, cudaStream_t s) {
   enum { K_INV = 0, K_LO = 1, K_UP = 2, K_BACK = 3, K_T = 4 };
   const int nx = L.cells[0];
   const long long n = L.N;
   const int t = nx / 2;
   auto rows = [&](int b) { return off[b + 1] - off[b]; };
   std::vector<long long> cpos(8 * (size_t)nx, -1);
-  long long ct = 0, maxe = 0;
+  long long ct = 0;
   for (int b = 0; b < nx; ++b) {
     const long long nb = rows(b), npv = b > 0 ? rows(b - 1) : 0, nnx = b + 1 < nx ? rows(b + 1) : 0;
     for (int sys = 0; sys < 2; ++sys) {
@@ -516,16 +438,13 @@ static stm_status twisted_slab_factors(Hierarchy& H, const Level& L, const std::
       if (b < t) { cpos[(k0 + K_BACK) * nx + b] = ct; ct += nb * nnx; }
       if (b > t) { cpos[(k0 + K_BACK) * nx + b] = ct; ct += nb * npv; }
     }
-    maxe = std::max(maxe, std::max(npv, nnx) * nb);
   }
-  double* E = nullptr;
-  if ((!H.cs_store && cudaMalloc(&H.cs_store, sizeof(double) * ct)) || cudaMalloc(&E, sizeof(double) * std::max(maxe, 1LL)) ||
+  if ((!H.cs_store && cudaMalloc(&H.cs_store, sizeof(double) * ct)) ||
       (!H.cs_u && cudaMalloc(&H.cs_u, sizeof(double) * n)) || (!H.cs_v && cudaMalloc(&H.cs_v, sizeof(double) * n)) ||
       (!H.cs_off && cudaMalloc(&H.cs_off, sizeof(long long) * (nx + 1))) ||
       (!H.cs_pos && cudaMalloc(&H.cs_pos, sizeof(long long) * 8 * nx)) ||
       (!H.cs_rowslab && cudaMalloc(&H.cs_rowslab, sizeof(int) * n)) || (!H.cs_perm && cudaMalloc(&H.cs_perm, sizeof(int) * n))) {
     cudaGetLastError();
-    if (E) cudaFree(E);
     set_error("coarse factorisation: out of device memory");
     return STM_ERR_OOM;
   }
@@ -534,45 +453,94 @@ static stm_status twisted_slab_factors(Hierarchy& H, const Level& L, const std::
   const double* D = raw;  // raw blocks: A_bb at dpos, A_{b,b-1} at lpos (b >= 1), A_{b,b+1} at upos (b < nx-1)
   auto Lo = [&](int b) { return D + lpos[b]; };
   auto Up = [&](int b) { return D + upos[b]; };
-  auto copy = [&](const double* src, long long r, long long c, double* dst) {
-    k_copy_block<<<(int)std::min<long long>((r * c + 255) / 256, sm_count() * 8LL), 256, 0, s>>>(src, r, c, c, dst, c);
-    note_launch();
-  };
   // one slab: S_b from A_bb and the neighbours already eliminated, its inverse, then its chain blocks
-  auto slab = [&](int b) {
-    const long long nb = rows(b), npv = b > 0 ? rows(b - 1) : 0, nnx = b + 1 < nx ? rows(b + 1) : 0;
+  auto slab = [&](int b, DenseWork& w, cudaStream_t st) -> stm_status {
+    const int nb = (int)rows(b), npv = b > 0 ? (int)rows(b - 1) : 0, nnx = b + 1 < nx ? (int)rows(b + 1) : 0;
     double* Sb = at(K_INV, b);
-    copy(D + dpos[b], nb, nb, Sb);
-    if (b > 0 && b <= t)  // - A_{b,b-1} W_{b-1}
-      dgemm((int)nb, (int)nb, (int)npv, -1.0, Lo(b), npv, at(K_BACK, b - 1), nb, 1.0, Sb, nb, s);
-    if (b + 1 < nx && b >= t)  // - A_{b,b+1} V_{b+1}
-      dgemm((int)nb, (int)nb, (int)nnx, -1.0, Up(b), nnx, at(K_BACK, b + 1), nb, 1.0, Sb, nb, s);
-    invert_block(Sb, nb, piv, scal, H.dflag + 1, maxsm, s);
-    if (b >= 1 && b <= t) dgemm((int)nb, (int)npv, (int)nb, 1.0, Sb, nb, Lo(b), npv, 0.0, at(K_LO, b), npv, s);
-    if (b >= t && b + 1 < nx) dgemm((int)nb, (int)nnx, (int)nb, 1.0, Sb, nb, Up(b), nnx, 0.0, at(K_UP, b), nnx, s);
-    if (b < t) dgemm((int)nb, (int)nnx, (int)nb, 1.0, Sb, nb, Up(b), nnx, 0.0, at(K_BACK, b), nnx, s);
-    if (b > t) dgemm((int)nb, (int)npv, (int)nb, 1.0, Sb, nb, Lo(b), npv, 0.0, at(K_BACK, b), npv, s);
-    // J_0^T: S_b^{-T}; (A_{b-1,b} S_b^{-1})^T and (A_{b+1,b} S_b^{-1})^T
-    transpose_block(Sb, nb, nb, at(K_T + K_INV, b), s);
+    const bool below = b > 0 && b <= t, above = b + 1 < nx && b >= t;  // neighbours already eliminated
+    const double* W = below ? at(K_BACK, b - 1) : nullptr;
+    const double* V = above ? at(K_BACK, b + 1) : nullptr;
+    const DenseSlice in[4] = {{2, false, below ? Lo(b) : nullptr, npv, below ? nb : 0, npv},
+                              {3, true, W, nb, below ? npv : 0, nb},
+                              {4, false, above ? Up(b) : nullptr, nnx, above ? nb : 0, nnx},
+                              {5, true, V, nb, above ? nnx : 0, nb}};
+    STM_TRY(dense_slice(w, in, 4, H.dflag + 1, st));
+    const double* cur = D + dpos[b];
+    DenseProduct p;
+    p.m = p.n = nb;
+    p.ldc0 = p.ldc = nb;
+    p.alpha = -1.0;
+    p.C = w.tmp;
+    if (below) {  // - A_{b,b-1} W_{b-1}
+      p.a = 2, p.b = 3, p.k = npv, p.C0 = cur;
+      STM_TRY(dense_products(w, &p, 1, st));
+      cur = w.tmp;
+    }
+    if (above) {  // - A_{b,b+1} V_{b+1}
+      p.a = 4, p.b = 5, p.k = nnx, p.C0 = cur;
+      STM_TRY(dense_products(w, &p, 1, st));
+      cur = w.tmp;
+    }
+    if (cur != w.tmp)
+      STM_CUDA(cudaMemcpyAsync(w.tmp, cur, sizeof(double) * (size_t)nb * nb, cudaMemcpyDeviceToDevice, st));
+    STM_TRY(invert_block(w, w.tmp, nb, Sb, H.dflag + 1, scal + 2 * (&w - H.dw), st));
+    // S_b^{-1} A_{b,b-1}, S_b^{-1} A_{b,b+1}; J_0^T: (A_{b-1,b} S_b^{-1})^T, (A_{b+1,b} S_b^{-1})^T, S_b^{-T}
+    const DenseSlice op[6] = {{0, false, Sb, nb, nb, nb},
+                              {1, true, Sb, nb, nb, nb},
+                              {2, true, b > 0 ? Lo(b) : nullptr, npv, npv ? nb : 0, npv},
+                              {3, true, b + 1 < nx ? Up(b) : nullptr, nnx, nnx ? nb : 0, nnx},
+                              {4, false, b > 0 ? Up(b - 1) : nullptr, nb, npv, nb},
+                              {5, false, b + 1 < nx ? Lo(b + 1) : nullptr, nb, nnx, nb}};
+    STM_TRY(dense_slice(w, op, 6, H.dflag + 1, st));
+    DenseProduct q[4];
+    int nq = 0;
+    auto product = [&](int a, int bb, int m, int n, double* C, int trans) {
+      DenseProduct& o = q[nq++];
+      o.a = a, o.b = bb, o.m = m, o.n = n, o.k = nb;
+      o.C = C, o.ldc = trans ? m : n, o.trans = trans;
+    };
     if (b > 0) {
-      dgemm((int)npv, (int)nb, (int)nb, 1.0, Up(b - 1), nb, Sb, nb, 0.0, E, nb, s);
-      transpose_block(E, npv, nb, at(K_T + (b <= t ? K_LO : K_BACK), b), s);
+      product(0, 2, nb, npv, at(b <= t ? K_LO : K_BACK, b), 0);
+      product(4, 1, npv, nb, at(K_T + (b <= t ? K_LO : K_BACK), b), 1);
     }
     if (b + 1 < nx) {
-      dgemm((int)nnx, (int)nb, (int)nb, 1.0, Lo(b + 1), nb, Sb, nb, 0.0, E, nb, s);
-      transpose_block(E, nnx, nb, at(K_T + (b < t ? K_BACK : K_UP), b), s);
+      product(0, 3, nb, nnx, at(b < t ? K_BACK : K_UP, b), 0);
+      product(5, 1, nnx, nb, at(K_T + (b < t ? K_BACK : K_UP), b), 1);
     }
+    STM_TRY(dense_products(w, q, nq, st));
+    transpose_block(Sb, nb, nb, at(K_T + K_INV, b), st);
+    return STM_OK;
   };
-  for (int b = 0; b < t; ++b) slab(b);
-  for (int b = nx - 1; b > t; --b) slab(b);
-  slab(t);
+  // the two chains meet only in slab t: the lower one runs on a stream of its own, with its own work space
+  long long maxnb = 0;
+  for (int b = 0; b < nx; ++b) maxnb = std::max(maxnb, rows(b));
+  for (DenseWork& w : H.dw) {
+    STM_TRY(dense_reserve_inverse(w, maxnb));
+    for (int q = 0; q < DenseWork::kSlots; ++q) STM_TRY(dense_reserve(w, q, maxnb, maxnb));
+  }
+  if (!H.chain_stream) STM_CUDA(cudaStreamCreateWithFlags(&H.chain_stream, cudaStreamNonBlocking));
+  for (cudaEvent_t& e : H.chain_ev)
+    if (!e) STM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  STM_CUDA(cudaEventRecord(H.chain_ev[0], s));
+  STM_CUDA(cudaStreamWaitEvent(H.chain_stream, H.chain_ev[0], 0));
+  stm_status chains = STM_OK;
+  for (int i = 0; i < std::max(t, nx - 1 - t) && chains == STM_OK; ++i) {
+    if (i < t) chains = slab(i, H.dw[0], s);
+    if (chains == STM_OK && nx - 1 - i > t) chains = slab(nx - 1 - i, H.dw[1], H.chain_stream);
+  }
+  STM_CUDA(cudaEventRecord(H.chain_ev[1], H.chain_stream));
+  STM_CUDA(cudaStreamWaitEvent(s, H.chain_ev[1], 0));
+  if (chains == STM_OK) chains = slab(t, H.dw[0], s);
+  if (chains != STM_OK) {
+    cudaStreamSynchronize(s);
+    return chains;
+  }
   std::vector<long long> hoff(off.begin(), off.begin() + nx + 1);
   cudaMemcpyAsync(H.cs_off, hoff.data(), sizeof(long long) * (nx + 1), cudaMemcpyHostToDevice, s);
   cudaMemcpyAsync(H.cs_pos, cpos.data(), sizeof(long long) * 8 * nx, cudaMemcpyHostToDevice, s);
   cudaMemcpyAsync(H.cs_rowslab, blk.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s);
   cudaMemcpyAsync(H.cs_perm, iperm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s);
   const cudaError_t e1 = cudaGetLastError(), e2 = cudaStreamSynchronize(s);
-  cudaFree(E);
   if (e1 != cudaSuccess || e2 != cudaSuccess) {
     set_error("coarse factorisation: CUDA error");
     return STM_ERR_CUDA;
@@ -608,17 +576,17 @@ stm_status factor_coarse(Hierarchy& H, cudaStream_t s) {
     if (b + 1 < nx) { wpos[b] = tot; tot += nb * (off[b + 2] - off[b + 1]); }
     if (b > 0) { gpos[b] = tot; tot += nb * (off[b] - off[b - 1]); }
   }
-  int *d_iperm = nullptr, *d_blk = nullptr, *piv = nullptr;
+  int *d_iperm = nullptr, *d_blk = nullptr;
   long long *d_off = nullptr, *d_dpos = nullptr, *d_lpos = nullptr, *d_upos = nullptr;
-  double *store = nullptr, *Xp = nullptr, *scal = nullptr;
+  double *Xp = nullptr, *scal = nullptr;
   stm_status st = STM_OK;
   auto fail = [&](stm_status e) { st = e; };
   do {
     if (cudaMalloc(&d_iperm, sizeof(int) * n) || cudaMalloc(&d_blk, sizeof(int) * n) ||
         cudaMalloc(&d_off, sizeof(long long) * (nx + 2)) || cudaMalloc(&d_dpos, sizeof(long long) * nx) ||
         cudaMalloc(&d_lpos, sizeof(long long) * nx) || cudaMalloc(&d_upos, sizeof(long long) * nx) ||
-        cudaMalloc(&store, sizeof(double) * tot) || (!use_slab && cudaMalloc(&Xp, sizeof(double) * n * n)) ||
-        cudaMalloc(&piv, sizeof(int) * maxnb) || cudaMalloc(&scal, sizeof(double) * 2)) {
+        (!H.cs_raw && cudaMalloc(&H.cs_raw, sizeof(double) * tot)) ||
+        (!use_slab && cudaMalloc(&Xp, sizeof(double) * n * n)) || cudaMalloc(&scal, sizeof(double) * 4)) {
       cudaGetLastError();
       set_error("coarse factorisation: out of device memory");
       fail(STM_ERR_OOM);
@@ -643,53 +611,77 @@ stm_status factor_coarse(Hierarchy& H, cudaStream_t s) {
     cudaMemcpyAsync(d_dpos, dpos.data(), sizeof(long long) * nx, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(d_lpos, lpos.data(), sizeof(long long) * nx, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(d_upos, upos.data(), sizeof(long long) * nx, cudaMemcpyHostToDevice, s);
+    double* store = H.cs_raw;
     cudaMemsetAsync(store, 0, sizeof(double) * tot, s);
     if (Xp) cudaMemsetAsync(Xp, 0, sizeof(double) * n * n, s);
     k_slab_blocks<<<(int)std::min<long long>(n, sm_count() * 32LL), 128, 0, s>>>(L.rowptr, L.colidx, L.val, n, d_iperm, d_blk,
                                                                           d_off, d_dpos, d_lpos, d_upos, store,
                                                                           H.dflag + 1);
     note_launch();
-    int dev = 0, maxsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (use_slab) {
-      st = twisted_slab_factors(H, L, off, iperm, blk, store, dpos, lpos, upos, piv, scal, maxsm, s);
+      st = twisted_slab_factors(H, L, off, iperm, blk, store, dpos, lpos, upos, scal, s);
       break;
     }
-    // forward block LU
-    for (int b = 0; b < nx; ++b) {
-      const long long nb = off[b + 1] - off[b];
-      double* Db = store + dpos[b];
-      if (b > 0) {  // S_b = A_bb - A_{b,b-1} W_{b-1}
-        const long long np_ = off[b] - off[b - 1];
-        dgemm((int)nb, (int)nb, (int)np_, -1.0, store + lpos[b], np_, store + wpos[b - 1], nb, 1.0, Db, nb, s);
+    // C (m x n) = [C0] + alpha A B, ld of each as given
+    DenseWork& w = H.dw[0];
+    auto product = [&](int m, int n_, int k, double alpha, const double* A, long long lda, const double* B, long long ldb,
+                       const double* C0, double* C, long long ldc) -> stm_status {
+      const DenseSlice sl[2] = {{2, false, A, lda, m, k}, {3, true, B, ldb, k, n_}};
+      STM_TRY(dense_slice(w, sl, 2, H.dflag + 1, s));
+      DenseProduct p;
+      p.a = 2, p.b = 3, p.m = m, p.n = n_, p.k = k, p.alpha = alpha;
+      p.C0 = C0, p.C = C, p.ldc0 = p.ldc = ldc;
+      return dense_products(w, &p, 1, s);
+    };
+    auto build = [&]() -> stm_status {
+      STM_TRY(dense_reserve_inverse(w, maxnb));
+      STM_TRY(dense_reserve(w, 2, maxnb, maxnb));
+      STM_TRY(dense_reserve(w, 3, maxnb, n));
+      // forward block LU
+      for (int b = 0; b < nx; ++b) {
+        const long long nb = off[b + 1] - off[b];
+        double* Db = store + dpos[b];
+        if (b > 0) {  // S_b = A_bb - A_{b,b-1} W_{b-1}
+          const long long np_ = off[b] - off[b - 1];
+          STM_TRY(product((int)nb, (int)nb, (int)np_, -1.0, store + lpos[b], np_, store + wpos[b - 1], nb, Db, w.tmp, nb));
+        } else {
+          STM_CUDA(cudaMemcpyAsync(w.tmp, Db, sizeof(double) * nb * nb, cudaMemcpyDeviceToDevice, s));
+        }
+        STM_TRY(invert_block(w, w.tmp, nb, Db, H.dflag + 1, scal, s));
+        if (b + 1 < nx) {  // W_b = S_b^{-1} A_{b,b+1}
+          const long long nn_ = off[b + 2] - off[b + 1];
+          STM_TRY(product((int)nb, (int)nn_, (int)nb, 1.0, Db, nb, store + upos[b], nn_, nullptr, store + wpos[b], nn_));
+        }
+        if (b > 0) {  // G_b = S_b^{-1} A_{b,b-1}
+          const long long np_ = off[b] - off[b - 1];
+          STM_TRY(product((int)nb, (int)np_, (int)nb, 1.0, Db, nb, store + lpos[b], np_, nullptr, store + gpos[b], np_));
+        }
       }
-      invert_block(Db, nb, piv, scal, H.dflag + 1, maxsm, s);
-      if (b + 1 < nx) {  // W_b = S_b^{-1} A_{b,b+1}
-        const long long nn_ = off[b + 2] - off[b + 1];
-        dgemm((int)nb, (int)nn_, (int)nb, 1.0, Db, nb, store + upos[b], nn_, 0.0, store + wpos[b], nn_, s);
+      // Z = L^{-1} (block lower triangular) into the block rows of Xp
+      for (int b = 0; b < nx; ++b) {
+        const long long nb = off[b + 1] - off[b];
+        double* rowb = Xp + off[b] * n;
+        k_copy_block<<<(int)std::min<long long>((nb * nb + 255) / 256, sm_count() * 8LL), 256, 0, s>>>(
+            store + dpos[b], nb, nb, nb, rowb + off[b], n);
+        note_launch();
+        if (b > 0) {
+          const long long np_ = off[b] - off[b - 1];
+          STM_TRY(product((int)nb, (int)off[b], (int)np_, -1.0, store + gpos[b], np_, Xp + off[b - 1] * n, n, nullptr,
+                          rowb, n));
+        }
       }
-      if (b > 0) {  // G_b = S_b^{-1} A_{b,b-1}
-        const long long np_ = off[b] - off[b - 1];
-        dgemm((int)nb, (int)np_, (int)nb, 1.0, Db, nb, store + lpos[b], np_, 0.0, store + gpos[b], np_, s);
+      // X = U^{-1} Z, last block row first
+      for (int b = nx - 2; b >= 0; --b) {
+        const long long nb = off[b + 1] - off[b], nn_ = off[b + 2] - off[b + 1];
+        STM_TRY(product((int)nb, (int)n, (int)nn_, -1.0, store + wpos[b], nn_, Xp + off[b + 1] * n, n, Xp + off[b] * n,
+                        Xp + off[b] * n, n));
       }
-    }
-    // Z = L^{-1} (block lower triangular) into the block rows of Xp
-    for (int b = 0; b < nx; ++b) {
-      const long long nb = off[b + 1] - off[b];
-      double* rowb = Xp + off[b] * n;
-      k_copy_block<<<(int)std::min<long long>((nb * nb + 255) / 256, sm_count() * 8LL), 256, 0, s>>>(
-          store + dpos[b], nb, nb, nb, rowb + off[b], n);
-      note_launch();
-      if (b > 0) {
-        const long long np_ = off[b] - off[b - 1];
-        dgemm((int)nb, (int)off[b], (int)np_, -1.0, store + gpos[b], np_, Xp + off[b - 1] * n, n, 0.0, rowb, n, s);
-      }
-    }
-    // X = U^{-1} Z, last block row first
-    for (int b = nx - 2; b >= 0; --b) {
-      const long long nb = off[b + 1] - off[b], nn_ = off[b + 2] - off[b + 1];
-      dgemm((int)nb, (int)n, (int)nn_, -1.0, store + wpos[b], nn_, Xp + off[b + 1] * n, n, 1.0, Xp + off[b] * n, n, s);
+      return STM_OK;
+    };
+    st = build();
+    if (st != STM_OK) {
+      cudaStreamSynchronize(s);
+      break;
     }
     dim3 ug((unsigned)std::min<long long>((n + 255) / 256, 64), (unsigned)std::min<long long>(n, 65535));
     k_unpermute<<<ug, 256, 0, s>>>(Xp, d_iperm, n, H.cinv);
@@ -700,7 +692,7 @@ stm_status factor_coarse(Hierarchy& H, cudaStream_t s) {
       fail(STM_ERR_CUDA);
     }
   } while (false);
-  void* ptrs[] = {d_iperm, d_blk, piv, d_off, d_dpos, d_lpos, d_upos, store, Xp, scal};
+  void* ptrs[] = {d_iperm, d_blk, d_off, d_dpos, d_lpos, d_upos, Xp, scal};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   return st;
