@@ -228,6 +228,16 @@ struct Level {
   double *d = nullptr, *r = nullptr, *t = nullptr;
   // multi-right-hand-side work space ([N][32] interleaved; mY: [C*n][32]), allocated on first use
   double *md = nullptr, *mr = nullptr, *mt = nullptr, *mY = nullptr;
+  // the 32-column product's operands (kernels_digit_spmm.cu): steps of 16 positions of node i from dbase[i],
+  // the velocity rows of J and J^T in fragment order with a power of two per row, X's words and bases
+  int* dbase = nullptr;           // [R+1]
+  long long dsteps = 0;
+  void* jw[2] = {};
+  int* jwexp[2] = {};
+  bool jw_current[2] = {};        // built from the present values
+  void* xw = nullptr;
+  short *xb = nullptr, *xnb = nullptr;  // bases of X, and the largest ones around every node
+  void* xmost = nullptr;
   uint32_t* mt16 = nullptr;       // [N][32] the smoothing step's residual block as packed BF16 (lo << 16 | hi)
 };
 
@@ -413,8 +423,12 @@ stm_status multi_columns_in(const double* src, double* dst, long long N, int nco
 stm_status multi_columns_out(const double* src, double* dst, long long N, int ncols, int col0, cudaStream_t s);
 // columns split..31 use J^T (L.valT, which must exist when split < 32)
 // T16 (mode 1 only, may be null): the result also as packed BF16 hi + lo parts (lo << 16 | hi)
-stm_status spmm_structured(const Level& L, const double* X, const double* B, double* Y, int mode, cudaStream_t s,
+stm_status spmm_structured(Level& L, const double* X, const double* B, double* Y, int mode, cudaStream_t s,
                            int split = 32, uint32_t* T16 = nullptr);
+// the same on the tensor cores, for up to six velocity rows per node (split 16 or 32)
+bool spmm_digits_supported(const Level& L);
+stm_status spmm_digits(Level& L, const double* X, const double* B, double* Y, int mode, cudaStream_t s, int split,
+                       uint32_t* T16);
 stm_status ensure_multi(Hierarchy& H);
 // split < 32: columns split..31 are adjoint columns (defect with J^T, local products with J_T^{-T});
 // with split = 16 and BF16 inverses on the tensor cores both come from one pass over the inverses

@@ -257,6 +257,7 @@ stm_status assemble_level(Hierarchy& H, int g, double nu, cudaStream_t s) {
                                          L.wnod, L.ref, L.ro, ac, L.dim, L.K, L.R, L.n, L.nt); note_launch();
     STM_CUDA(cudaGetLastError());
   }
+  L.jw_current[0] = L.jw_current[1] = false;
   if (L.valT) {
     cudaFree(L.valT);
     L.valT = nullptr;

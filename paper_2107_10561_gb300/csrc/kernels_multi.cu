@@ -1,8 +1,9 @@
 // Multi-right-hand-side path: up to 32 right-hand sides share one hierarchy (one J, one set of
 // cell inverses). Multi-vectors are stored interleaved, [N][32] FP64 (column c of DoF i at
 // i * 32 + c), so every gather of a DoF fetches its 32 values in one 256-byte line.
-//  * SpMM with J_g: the structured pattern of k_spmv_struct, one warp per node (cell) with the
-//    32 lanes on the 32 right-hand sides: each value of J is read once for all columns (broadcast).
+//  * SpMM with J_g: on the tensor cores over base-256 digits (kernels_digit_spmm.cu); with more than six
+//    velocity rows per node (3D dG(2)) here in FP64, one warp per node (cell) with the 32 lanes on the
+//    32 right-hand sides: each value of J is read once for all columns (broadcast).
 //  * Vanka local solves Y_T = J_T^{-1} T_T for a 32-column block (a6'' of the hot path): with BF16
 //    inverses on the tcgen05 tensor cores (kernels_mrhs_tc.cu: TMA-staged inverses, FP32 accumulators
 //    in tensor memory, the gathered block split into T_hi + T_lo BF16 parts so that the only rounding
@@ -191,12 +192,13 @@ __global__ void __launch_bounds__(256) k_spmm_struct(
   }
 }
 
-stm_status spmm_structured(const Level& L, const double* X, const double* B, double* Y, int mode, cudaStream_t s,
-                           int split, uint32_t* T16) {
+stm_status spmm_structured(Level& L, const double* X, const double* B, double* Y, int mode, cudaStream_t s, int split,
+                           uint32_t* T16) {
   if (split < NR && !L.valT) {
     set_error("multi-RHS SpMM: the values of J^T are not built");
     return STM_ERR_STATE;
   }
+  if (spmm_digits_supported(L)) return spmm_digits(L, X, B, Y, mode, s, split, T16);
   const long long jobs = (long long)L.R + L.C;
   const int blocks = (int)std::min<long long>((jobs * 32 + 255) / 256, (long long)msms() * 8);
   const int key = L.dim * 10 + L.K;
@@ -204,12 +206,7 @@ stm_status spmm_structured(const Level& L, const double* X, const double* B, dou
   k_spmm_struct<K, D><<<blocks, 256, 0, s>>>(L.rowptr, L.val, L.nbr_ptr, L.nbr, L.ncell, L.node_cells, L.cell_nodes, \
                                              L.block, L.R, L.C, L.nv, X, B, Y, mode, L.valT, split, T16)
   switch (key) {
-    case 21: SPMM(1, 2); break;
-    case 22: SPMM(2, 2); break;
-    case 23: SPMM(3, 2); break;
-    case 31: SPMM(1, 3); break;
-    case 32: SPMM(2, 3); break;
-    case 33: SPMM(3, 3); break;
+    case 33: SPMM(3, 3); break;  // nine rows per node
     default:
       set_error("multi-RHS SpMM: unsupported (dim, k)");
       return STM_ERR_INVALID_ARG;
