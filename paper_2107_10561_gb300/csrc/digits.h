@@ -70,4 +70,59 @@ __device__ __forceinline__ double scale_pow2(double v, int e) {
   return ldexp(v, e);
 }
 
+// Sums of fewer than 2^22 in magnitude may start from kSumZero: 1.5 x 2^23, so that the sum's integer stands in
+// the low bits of the FP32 pattern (a conversion would run at an eighth of the FMA rate).
+constexpr float kSumZero = 12582912.f;
+// hi (digits 0 .. 3) and lo (4 .. 7) of eight such sums: sum_d s_d 256^(3 - d)
+__device__ __forceinline__ void join_sums(const float (*acc)[4], int m, long long& hi, long long& lo) {
+  constexpr long long zero = 0x4B400000ll * (16777216 + 65536 + 256 + 1);
+  hi = lo = -zero;
+#pragma unroll
+  for (int d = 0; d < 4; ++d) {
+    hi += (long long)__float_as_int(acc[d][m]) * (1 << (24 - 8 * d));
+    lo += (long long)__float_as_int(acc[d + 4][m]) * (1 << (24 - 8 * d));
+  }
+}
+// (hi * 2^32 + lo) * 2^e, rounded once, with integer operations only: conversions and products would wait for
+// the FP64 pipe. |hi| < 2^62.
+__device__ __forceinline__ double join_pow2(long long hi, long long lo, int e) {
+  long long h = hi + (lo >> 32);
+  uint32_t l = (uint32_t)lo;  // the value is h * 2^32 + l
+  const bool neg = h < 0;
+  if (neg) {
+    h = l ? ~h : -h;
+    l = 0u - l;
+  }
+  unsigned long long u = (unsigned long long)h;
+  if (u == 0) {
+    if (l == 0) return 0.0;
+    u = l;
+    l = 0;
+    e -= 32;
+  }
+  const int lz = __clzll((long long)u), ex = 1023 + 63 + 32 - lz + e;
+  u = (u << lz) | (((unsigned long long)l << 32) >> (64 - lz));  // lz >= 1
+  if (ex < 1 || ex > 2045) {
+    const double v = scale_pow2((double)u, 32 - lz + e);
+    return neg ? -v : v;
+  }
+  u = (u >> 11) + ((u >> 10) & 1);  // 53 bits, the rounding may carry into the exponent
+  u += ((unsigned long long)(ex - 1) << 52);
+  return __longlong_as_double((long long)(u | (neg ? 0x8000000000000000ull : 0ull)));
+}
+// |v| as an integer key that orders like |v|; NaN orders below everything
+__device__ __forceinline__ long long abs_key(double v) {
+  const long long k = __double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll;
+  return k > 0x7FF0000000000000ll ? -1 : k;
+}
+// 1 / a: the hardware's approximation and two Newton steps, four dependent FP64 operations
+__device__ __forceinline__ double reciprocal(double a) {
+  const int ex = (__double2hiint(a) >> 20) & 0x7FF;
+  if (ex < 64 || ex > 1982) return 1.0 / a;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+  r = fma(r, fma(-a, r, 1.0), r);
+  return fma(r, fma(-a, r, 1.0), r);
+}
+
 }  // namespace stm

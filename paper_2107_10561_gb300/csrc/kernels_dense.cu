@@ -12,6 +12,7 @@
 // tiles) and 0.035 ms for cutting both operands, against 3.3 ms for a tiled FP64 kernel; error 6e-17
 // |A||B| against 1.3e-15 of an FMA chain.
 #include <cfloat>
+#include <climits>
 
 #include "digits.h"
 #include "internal.h"
@@ -26,7 +27,7 @@ constexpr int kRowB = 112;         // bytes of one k-row of B in shared memory (
 constexpr int kStageA = kDig * kTileM * kTileK * 2;  // 32 KB
 constexpr int kStageB = kDig * kTileK * kRowB;       // 28 KB
 constexpr int kPanel = 32;   // pivots per panel of the blocked inverse
-constexpr int kSmallInv = 192;  // up to this size one panel is the whole matrix
+constexpr int kSmallInv = 128;  // up to this size one panel is the whole matrix (144 rows: 0.37 ms against 0.30 blocked)
 constexpr int kCluster = 16;
 constexpr int kPanelRows = 512;    // panel rows per CTA at most: 32 columns fill 130 KB
 
@@ -268,67 +269,100 @@ __device__ __forceinline__ uint32_t cluster_rank() {
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void remote_store(uint32_t addr, uint32_t rank, double v) {
-  uint32_t ra;
+// Asynchronous 16-byte store into the shared memory of another CTA of the cluster, counted by its barrier.
+__device__ __forceinline__ void remote_store(uint32_t addr, uint32_t bar, uint32_t rank, double v0, double v1) {
+  uint32_t ra, rb;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(v) : "memory");
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(bar), "r"(rank));
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(ra),
+               "l"(__double_as_longlong(v0)), "l"(__double_as_longlong(v1)), "r"(rb)
+               : "memory");
 }
-__device__ __forceinline__ void remote_store(uint32_t addr, uint32_t rank, int v) {
-  uint32_t ra;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
-  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(ra), "r"(v) : "memory");
+__device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// Waits for the barrier's phase for one second at most; false if it did not come.
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
+  uint32_t done = 0;
+  unsigned long long t0 = 0;
+  for (int i = 0;; ++i) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    if (done) return true;
+    if ((i & 255) == 255) {
+      unsigned long long t;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > 1000000000ull) return false;
+    }
+  }
+}
+// Lane (of `lanes`) with the largest key, the smallest row among equal keys; every lane of the warp calls.
+__device__ __forceinline__ int best_lane(long long key, int row, int lanes) {
+  const int lane = threadIdx.x & 31;
+  const int hi = lane < lanes ? (int)(key >> 32) : INT_MIN;  // keys are >= -1
+  const int mh = __reduce_max_sync(0xffffffffu, hi);
+  unsigned m = __ballot_sync(0xffffffffu, hi == mh);
+  if (m & (m - 1)) {
+    const unsigned lo = hi == mh ? (unsigned)key : 0u;
+    const unsigned ml = __reduce_max_sync(0xffffffffu, lo);
+    m = __ballot_sync(0xffffffffu, hi == mh && (unsigned)key == ml);
+    if (m & (m - 1)) {
+      const int r = (m >> lane) & 1u ? row : INT_MAX;
+      const int mr = __reduce_min_sync(0xffffffffu, r);
+      m = __ballot_sync(0xffffffffu, ((m >> lane) & 1u) && row == mr);
+    }
+  }
+  return __ffs(m) - 1;
 }
 
-// Row pitch of the panel in shared memory (odd, so that a column is read without bank conflicts) and the
-// shared memory of one CTA: its rows, two mailboxes (every CTA's candidate row, the row to be exchanged, the
-// candidates' keys, rows and reciprocals) and the warps' candidates.
+// Row pitch of the panel in shared memory (odd, so that a column is read without bank conflicts), pitch of the
+// rows that are sent (even: 16-byte pieces), and the shared memory of one CTA: two mailboxes (every CTA's
+// candidate row, the row to be exchanged, the candidates' keys, reciprocals and rows), its rows, the warps'
+// candidates.
 __host__ __device__ inline int panel_pitch(int w) { return w | 1; }
-__host__ __device__ inline size_t panel_smem(int rpc, int w) {
-  return sizeof(double) * ((size_t)rpc * panel_pitch(w) + 2 * (size_t)(kCluster + 1) * w) +
-         2 * kCluster * (sizeof(long long) + sizeof(double) + sizeof(int)) + 8 * (sizeof(long long) + sizeof(int));
-}
-// |v| as an integer key that orders like |v|; NaN orders below everything
-__device__ __forceinline__ long long abs_key(double v) {
-  const long long k = __double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll;
-  return k > 0x7FF0000000000000ll ? -1 : k;
-}
-// 1 / a: the hardware's approximation and two Newton steps, four dependent FP64 operations
-__device__ __forceinline__ double reciprocal(double a) {
-  const int ex = (__double2hiint(a) >> 20) & 0x7FF;
-  if (ex < 64 || ex > 1982) return 1.0 / a;
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-  r = fma(r, fma(-a, r, 1.0), r);
-  return fma(r, fma(-a, r, 1.0), r);
+__host__ __device__ inline int mail_pitch(int w) { return (w + 1) & ~1; }
+__host__ __device__ inline size_t mail_doubles(int nc, int w) { return (size_t)(nc + 1) * mail_pitch(w) + 4 * nc; }
+__host__ __device__ inline size_t panel_smem(int nc, int rpc, int w) {
+  return sizeof(double) * (2 * mail_doubles(nc, w) + (size_t)rpc * panel_pitch(w)) + 8 * (sizeof(long long) + sizeof(int));
 }
 
 // In-place Gauss-Jordan on columns [k0, k0 + w) of the n x n matrix A, rows kept in the shared memory of
 // one 16-CTA cluster. Pivot k is the largest entry of column k0 + k among rows >= k0 + k (lowest row on
-// ties). Each CTA pushes its best row and that row's reciprocal pivot into every CTA's mailbox before the
-// one cluster barrier of the pivot, so the winner is known and at hand everywhere after it. The panel ends
-// as the block transform M: any other column c becomes (c with the panel's rows cleared) + M c_panel after
-// the row exchanges. What bounds it: an FP64 instruction occupies its pipe for 64 clocks, so per pivot the
-// update (one FMA per row and 32 columns), the reciprocal and the barrier follow one another; keys are
-// compared as integers, and the next pivot's candidates are taken while the rows are updated. With digits
-// set, M is also written as a row operand of the digit product (w <= 32 only). Measured: 5.1 ms for the
-// inverse of a 1125 x 1125 block (36 panels of 32), 0.27 ms at 99 x 99 (one panel), against 34 ms with one
-// pivot per four launches and 1.23 ms for a Gauss-Jordan in one CTA's shared memory.
-template <int Q>  // 32-column blocks: w <= 32 Q
+// ties). Each CTA sends its best row with that row's key and reciprocal pivot to every CTA, by asynchronous
+// stores that the receivers' barriers count, so a pivot costs one flight between CTAs and no cluster-wide
+// barrier: a CTA goes on when all sixteen have sent. (It cannot run more than one pivot ahead of any other,
+// so two mailboxes are enough.) The panel ends as the block transform M: any other column c becomes (c with
+// the panel's rows cleared) + M c_panel after the row exchanges. What bounds it: the flight, and an FP64
+// instruction that occupies its pipe for 64 clocks (one FMA per row and 32 columns); keys are compared as
+// integers, and the next pivot's candidates are taken while the rows are updated. With words set, M is
+// also written as the row operand of the update (w <= 32 only). Measured: 1.3 us per pivot at 32 rows (with a
+// cluster barrier per pivot 1.8 us), 0.16 ms for a whole 96 x 96 block; blocked inverse of 1125 rows 3.7 ms,
+// against 34 ms with one pivot per four launches and 1.23 ms at 99 rows for one CTA's shared memory.
+template <int Q, int NC>  // 32-column blocks: w <= 32 Q; CTAs of the cluster
 __global__ void __launch_bounds__(256) k_gj_panel(double* __restrict__ A, int n, int k0, int w, int* __restrict__ piv,
-                                                  int* flag, __half* __restrict__ dig, long long plane,
-                                                  int* __restrict__ exps) {
+                                                  int* flag, uint4* __restrict__ words, int* __restrict__ exps) {
   extern __shared__ __align__(16) double sd[];
+  __shared__ __align__(8) unsigned long long bars[2];
+  __shared__ int s_late;
   const int rank = (int)cluster_rank();
-  const int rpc = (n + kCluster - 1) / kCluster, ws = panel_pitch(w);
+  const int rpc = (n + NC - 1) / NC, ws = panel_pitch(w), wp = mail_pitch(w);
   const int r0 = min(rank * rpc, n), r1 = min(r0 + rpc, n), nr = r1 - r0;
-  double* P = sd;                          // [rpc][ws]
-  double* mail = P + (size_t)rpc * ws;     // [2][17][w]: candidate rows, then row k0 + k
-  long long* ckey = reinterpret_cast<long long*>(mail + 2 * (size_t)(kCluster + 1) * w);  // [2][16]
-  double* cinv = reinterpret_cast<double*>(ckey + 2 * kCluster);                           // [2][16]
-  long long* wkey = reinterpret_cast<long long*>(cinv + 2 * kCluster);                     // [8]
-  int* cidx = reinterpret_cast<int*>(wkey + 8);                                            // [2][16]
-  int* widx = cidx + 2 * kCluster;                                                         // [8]
+  // a mailbox: [16][wp] candidate rows, [wp] row k0 + k, [16][2] key and reciprocal, [16][2] row
+  const size_t box_len = mail_doubles(NC, w);
+  double* P = sd + 2 * box_len;            // [rpc][ws]
+  long long* wkey = reinterpret_cast<long long*>(P + (size_t)rpc * ws);  // [8]
+  int* widx = reinterpret_cast<int*>(wkey + 8);                          // [8]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t bytes = (uint32_t)(NC * (wp * 8 + 32) + wp * 8);  // received per pivot
+  if (tid == 0) {
+    s_late = 0;
+    for (int i = 0; i < 2; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bars + i)));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
   // candidate of this warp's rows for column k0 (later columns: while the rows are updated)
   long long bk = -1;
   int bi = n;
@@ -352,50 +386,51 @@ __global__ void __launch_bounds__(256) k_gj_panel(double* __restrict__ A, int n,
   cluster_sync();
   for (int k = 0; k < w; ++k) {
     const int gk = k0 + k, buf = k & 1;
-    double* box = mail + (size_t)buf * (kCluster + 1) * w;
+    double* box = sd + buf * box_len;
+    const uint32_t bar = smem_addr(bars + buf);
     // this CTA's candidate: every warp takes the best of the eight (lowest row on ties)
-    bk = wkey[lane & 7];
-    bi = widx[lane & 7];
-#pragma unroll
-    for (int off = 4; off > 0; off >>= 1) {
-      const long long ok = __shfl_xor_sync(0xffffffffu, bk, off);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-      if (ok > bk || (ok == bk && oi < bi)) { bk = ok; bi = oi; }
+    {
+      const long long key = wkey[lane & 7];
+      const int row = widx[lane & 7], l = best_lane(key, row, 8);
+      bk = __shfl_sync(0xffffffffu, key, l);
+      bi = __shfl_sync(0xffffffffu, row, l);
     }
-    const bool mine = gk >= r0 && gk < r1;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int j = 32 * q + lane;
-      const double cand = bk >= 0 && j < w ? P[(size_t)(bi - r0) * ws + j] : 0.0;
-      const double old = mine && j < w ? P[(size_t)(gk - r0) * ws + j] : 0.0;
-      if (j < w)
-#pragma unroll
-        for (int d = 0; d < kCluster; d += 8) {
-          if (bk >= 0) remote_store(smem_addr(box + (size_t)rank * w + j), d + warp, cand);
-          if (mine) remote_store(smem_addr(box + (size_t)kCluster * w + j), d + warp, old);
-        }
-    }
-    if (warp == 7) {
+    if (warp == 7) {  // the reciprocal takes longest
       const double inv = bk >= 0 ? reciprocal(P[(size_t)(bi - r0) * ws + k]) : 0.0;
-      if (lane < kCluster) {
-        remote_store(smem_addr(ckey + buf * kCluster + rank), lane, __longlong_as_double(bk));
-        remote_store(smem_addr(cinv + buf * kCluster + rank), lane, inv);
-        remote_store(smem_addr(cidx + buf * kCluster + rank), lane, bi);
+      const uint32_t at = smem_addr(box + (size_t)(NC + 1) * wp + 2 * rank);
+      if (lane < NC) remote_store(at, bar, lane, __longlong_as_double(bk), inv);
+      else if (lane < 2 * NC) remote_store(at + 16 * NC, bar, lane - NC, __longlong_as_double(bi), 0.0);
+      if (lane == 0) bar_expect(bar, bytes);
+    } else {
+      const bool mine = gk >= r0 && gk < r1;
+      const int h = wp >> 1;  // 16-byte pieces of a row
+      for (int e = tid; e < NC * h; e += 224) {
+        const int d = Q == 1 && w == 32 ? e >> 4 : e / h, j = 2 * (e - d * h);
+        double c0 = 0.0, c1 = 0.0;
+        if (bk >= 0) {
+          c0 = P[(size_t)(bi - r0) * ws + j];
+          if (j + 1 < w) c1 = P[(size_t)(bi - r0) * ws + j + 1];
+        }
+        remote_store(smem_addr(box + (size_t)rank * wp + j), bar, d, c0, c1);
+        if (mine) {
+          const double o0 = P[(size_t)(gk - r0) * ws + j], o1 = j + 1 < w ? P[(size_t)(gk - r0) * ws + j + 1] : 0.0;
+          remote_store(smem_addr(box + (size_t)NC * wp + j), bar, d, o0, o1);
+        }
       }
     }
-    cluster_sync();
-    bk = ckey[buf * kCluster + (lane & 15)];
-    bi = cidx[buf * kCluster + (lane & 15)];
-    int who = lane & 15;
-#pragma unroll
-    for (int off = 8; off > 0; off >>= 1) {
-      const long long ok = __shfl_xor_sync(0xffffffffu, bk, off);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-      const int ow = __shfl_xor_sync(0xffffffffu, who, off);
-      if (ok > bk || (ok == bk && oi < bi)) { bk = ok; bi = oi; who = ow; }
+    if (!bar_wait(bar, (k >> 1) & 1)) s_late = 1;
+    const double* cand = box + (size_t)(NC + 1) * wp;
+    int who;
+    {
+      const long long key = __double_as_longlong(cand[2 * (lane & (NC - 1))]);
+      const int row = (int)__double_as_longlong(cand[2 * NC + 2 * (lane & (NC - 1))]);
+      who = best_lane(key, row, NC);
+      bk = __shfl_sync(0xffffffffu, key, who);
+      bi = __shfl_sync(0xffffffffu, row, who);
     }
     const int p = bi;
-    if (bk <= 0 || bk >= 0x7FF0000000000000ll) {  // the same decision in every CTA of the cluster
+    // the same decision in every CTA of the cluster
+    if (bk <= 0 || bk >= 0x7FF0000000000000ll) {
       if (rank == 0 && tid == 0) {
         atomicExch(flag, 1);
         for (int q = k; q < w; ++q) piv[k0 + q] = k0 + q;
@@ -403,9 +438,9 @@ __global__ void __launch_bounds__(256) k_gj_panel(double* __restrict__ A, int n,
       break;
     }
     if (rank == 0 && tid == 0) piv[gk] = p;
-    const double* prow = box + (size_t)who * w;
-    const double* krow = box + (size_t)kCluster * w;
-    const double pinv = cinv[buf * kCluster + who];
+    const double* prow = box + (size_t)who * wp;
+    const double* krow = box + (size_t)NC * wp;
+    const double pinv = cand[2 * who + 1];
     // one warp per row, lanes over the columns: row p takes the old row k0 + k, row k0 + k the scaled
     // pivot row, every other row loses its multiple of it; column k becomes the transform's column
     // (0 - f pinv), so one FMA serves all columns
@@ -445,6 +480,11 @@ __global__ void __launch_bounds__(256) k_gj_panel(double* __restrict__ A, int n,
       widx[warp] = bi;
     }
     __syncthreads();
+    if (s_late) {  // a CTA that does not hear from the others gives up, and then they do
+      if (tid == 0) atomicExch(flag, 1);
+      for (int q = k + 1 + tid; rank == 0 && q < w; q += 256) piv[k0 + q] = k0 + q;
+      break;
+    }
   }
   for (int i = warp; i < nr; i += 8)
 #pragma unroll
@@ -452,28 +492,33 @@ __global__ void __launch_bounds__(256) k_gj_panel(double* __restrict__ A, int n,
       const int j = 32 * q + lane;
       if (j < w) A[(long long)(r0 + i) * n + k0 + j] = P[(size_t)i * ws + j];
     }
-  if (Q == 1 && dig) {
+  if (Q == 1 && words) {  // [16-row tile][16 positions][4][32 lanes], two neighbouring positions per word set
     for (int i = warp; i < nr; i += 8) {
+      const int r = r0 + i;
       const double v = lane < w ? P[(size_t)i * ws + lane] : 0.0;
-      int e = exp_above(v);
-      for (int off = 16; off > 0; off >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
+      const int e = __reduce_max_sync(0xffffffffu, exp_above(v));
       const bool bad = e > 1024;
       if (bad && lane == 0) atomicExch(flag, 1);
       const unsigned long long pk = digits_of(bad ? 0.0 : v, e);
-#pragma unroll
-      for (int d = 0; d < kDig; ++d) dig[d * plane + (long long)(r0 + i) * kPanel + lane] = digit_half(pk, d);
-      if (lane == 0) exps[r0 + i] = e;
+      const unsigned long long nx = __shfl_down_sync(0xffffffffu, pk, 1);
+      if (!(lane & 1)) {
+        const int pp = lane >> 1;
+        words[((r >> 4) * 2 + (pp >> 3)) * 128 + (((r >> 3) & 1) + 2 * ((pp >> 2) & 1)) * 32 + (r & 7) * 4 + (pp & 3)] =
+            words_of(pk, nx);
+      }
+      if (lane == 0) exps[r] = e;
     }
   }
   cluster_sync();  // no CTA leaves while another may still write into its mailbox
 }
 
-// The row exchanges of one panel on every other column, the panel's rows as a column operand of the digit
-// product (scaled per column), and zeros in their place. One thread per column; the exchanges are first
-// composed into source rows, so that all loads of a column are independent.
+// The row exchanges of one panel on the columns [c0, c1) without the panel's own and without [x0, x1), and the
+// panel's rows as the column operand of the update ([pair][column] word sets, scaled per column). One thread
+// per column; the exchanges are first composed into source rows, so that all loads of a column are
+// independent.
 __global__ void __launch_bounds__(128) k_gj_rows(double* __restrict__ A, int n, int k0, int w, const int* __restrict__ piv,
-                                                 int* flag, __half* __restrict__ dig, long long plane, int pitch,
-                                                 int* __restrict__ exps) {
+                                                 int c0, int c1, int x0, int x1, int* flag, uint4* __restrict__ words,
+                                                 int pitch, int* __restrict__ exps) {
   extern __shared__ int at[];  // at[r]: row that now sits at r
   for (int r = threadIdx.x; r < n; r += 128) at[r] = r;
   __shared__ int dst[kPanel], src[kPanel], top[kPanel];
@@ -494,14 +539,13 @@ __global__ void __launch_bounds__(128) k_gj_rows(double* __restrict__ A, int n, 
     src[k] = out ? at[p] : k0;
   }
   __syncthreads();
-  const int j = blockIdx.x * 128 + threadIdx.x;
-  if (j >= pitch) return;
-  const bool live = j < n && (j < k0 || j >= k0 + w);
+  const int j = c0 + blockIdx.x * 128 + threadIdx.x;
+  if (j >= c1 || (j >= k0 && j < k0 + w) || (j >= x0 && j < x1)) return;
   double v[kPanel], t[kPanel];
 #pragma unroll
   for (int k = 0; k < kPanel; ++k) {
-    v[k] = live && k < w ? A[(long long)top[k] * n + j] : 0.0;
-    t[k] = live && dst[k] >= 0 ? A[(long long)src[k] * n + j] : 0.0;
+    v[k] = k < w ? A[(long long)top[k] * n + j] : 0.0;
+    t[k] = dst[k] >= 0 ? A[(long long)src[k] * n + j] : 0.0;
   }
   int e = kExpZero;
 #pragma unroll
@@ -509,17 +553,87 @@ __global__ void __launch_bounds__(128) k_gj_rows(double* __restrict__ A, int n, 
   const bool bad = e > 1024;
   if (bad) atomicExch(flag, 1);
 #pragma unroll
-  for (int k = 0; k < kPanel; ++k) {
-    if (live && k < w) A[(long long)(k0 + k) * n + j] = 0.0;
-    if (live && dst[k] >= 0) A[(long long)dst[k] * n + j] = t[k];
-  }
+  for (int k = 0; k < kPanel; ++k)
+    if (dst[k] >= 0) A[(long long)dst[k] * n + j] = t[k];
 #pragma unroll
-  for (int k = 0; k < kPanel; ++k) {
-    const unsigned long long pk = digits_of(bad ? 0.0 : v[k], e);
+  for (int k = 0; k < kPanel; k += 2)
+    words[(long long)(k >> 1) * pitch + j] = words_of(digits_of(bad ? 0.0 : v[k], e), digits_of(bad ? 0.0 : v[k + 1], e));
+  exps[j] = e;
+}
+
+constexpr int kUpCols = 48;  // columns per warp of the update
+
+// C = (C with the panel's rows cleared) + M R on the columns [c0, c1) without the panel's own and without [x0, x1): a
+// warp takes 16 rows and 48 columns with M's digits in registers; the next eight columns' operands and
+// entries are loaded while the present ones are multiplied. At 1125 rows that is one wave of twelve warps
+// per SM.
+__global__ void __launch_bounds__(128, 3) k_gj_update(double* __restrict__ A, int n, int k0, int w,
+                                                      const uint4* __restrict__ mw, const int* __restrict__ em,
+                                                      const uint4* __restrict__ rw, const int* __restrict__ er, int pitch,
+                                                      int c0, int c1, int x0, int x1) {
+  const int lane = threadIdx.x & 31, nq = lane >> 2, q = lane & 3;
+  const int groups = (c1 - c0 + kUpCols - 1) / kUpCols, tiles = (n + 15) / 16;
+  const int un = blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (un >= groups * tiles) return;
+  const int mt = un / groups, j0 = c0 + (un - mt * groups) * kUpCols, j1 = min(j0 + kUpCols, c1);
+  uint32_t a[2][kDig][4];
 #pragma unroll
-    for (int d = 0; d < kDig; ++d) dig[d * plane + (long long)k * pitch + j] = digit_half(pk, d);
+  for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint4 x = __ldg(mw + (mt * 2 + kk) * 128 + k * 32 + lane);
+      const uint32_t xx[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int d = 0; d < kDig; ++d) a[kk][d][k] = digit_pair(xx[d & 3], d >= 4);
+    }
+  const int r0 = 16 * mt + nq, e0 = em[min(r0, n - 1)], e8 = em[min(r0 + 8, n - 1)];
+  auto live = [&](int j) { return j < j1 && (j < k0 || j >= k0 + w) && (j < x0 || j >= x1); };
+  uint4 nx[4];
+  double nc[4];
+  auto load = [&](int jb) {
+    const int jc = min(jb + nq, c1 - 1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) nx[k] = __ldg(rw + (long long)(4 * k + q) * pitch + jc);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const int r = r0 + (m < 2 ? 0 : 8), j = jb + 2 * q + (m & 1);
+      nc[m] = r < n && live(j) && (r < k0 || r >= k0 + w) ? A[(long long)r * n + j] : 0.0;
+    }
+  };
+  load(j0);
+#pragma unroll 1
+  for (int jb = j0; jb < j1; jb += 8) {
+    uint4 y[4] = {nx[0], nx[1], nx[2], nx[3]};
+    double cv[4] = {nc[0], nc[1], nc[2], nc[3]};
+    if (jb + 8 < j1) load(jb + 8);
+    float acc[kDig][4];
+#pragma unroll
+    for (int d = 0; d < kDig; ++d)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) acc[d][m] = kSumZero;
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk) {
+      const uint32_t y0[4] = {y[2 * kk].x, y[2 * kk].y, y[2 * kk].z, y[2 * kk].w};
+      const uint32_t y1[4] = {y[2 * kk + 1].x, y[2 * kk + 1].y, y[2 * kk + 1].z, y[2 * kk + 1].w};
+#pragma unroll
+      for (int o = 0; o < kDig; ++o) {
+        const uint32_t b0 = digit_pair(y0[o & 3], o >= 4), b1 = digit_pair(y1[o & 3], o >= 4);
+#pragma unroll
+        for (int d = 0; d + o < kDig; ++d) mma_f16(acc[d + o], a[kk][d][0], a[kk][d][1], a[kk][d][2], a[kk][d][3], b0, b1);
+      }
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const int r = r0 + (m < 2 ? 0 : 8), j = jb + 2 * q + (m & 1);
+      if (r >= n || !live(j)) continue;
+      // sums of 8 pairs x 32 terms, products at most 2^14 (2^13 where a leading digit takes part)
+      long long hi, lo;
+      join_sums(acc, m, hi, lo);
+      const int ea = m < 2 ? e0 : e8, eb = er[j];
+      if (ea != kExpZero && eb != kExpZero) cv[m] += join_pow2(hi, lo, ea + eb - 124 + 56);
+      A[(long long)r * n + j] = cv[m];
+    }
   }
-  if (j < n) exps[j] = e;
 }
 
 // Undo the row exchanges as column exchanges, last first: out[:, j] = A[:, from[j]].
@@ -549,24 +663,23 @@ int up(int v, int m) { return (v + m - 1) / m * m; }
 
 constexpr int kMaxCluster = kCluster * kPanelRows;  // rows of the largest block inverted by clusters
 
-template <int Q>
-stm_status launch_panel(double* A, int n, int k0, int w, int* piv, int* flag, __half* dig, long long plane, int* exps,
-                        cudaStream_t s) {
-  const size_t smem = panel_smem((n + kCluster - 1) / kCluster, w);
-  STM_CUDA(cudaFuncSetAttribute(k_gj_panel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  STM_CUDA(cudaFuncSetAttribute(k_gj_panel<Q>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+template <int Q, int NC>
+stm_status launch_panel(double* A, int n, int k0, int w, int* piv, int* flag, uint4* words, int* exps, cudaStream_t s) {
+  const size_t smem = panel_smem(NC, (n + NC - 1) / NC, w);
+  STM_CUDA(cudaFuncSetAttribute(k_gj_panel<Q, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  STM_CUDA(cudaFuncSetAttribute(k_gj_panel<Q, NC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(kCluster);
+  cfg.gridDim = dim3(NC);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = kCluster;
+  at.val.clusterDim.x = NC;
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  STM_CUDA(cudaLaunchKernelEx(&cfg, k_gj_panel<Q>, A, n, k0, w, piv, flag, dig, plane, exps));
+  STM_CUDA(cudaLaunchKernelEx(&cfg, k_gj_panel<Q, NC>, A, n, k0, w, piv, flag, words, exps));
   note_launch();
   return STM_OK;
 }
@@ -602,8 +715,9 @@ stm_status dense_reserve(DenseWork& w, int slot, long long rows, long long cols)
 }
 
 stm_status dense_reserve_inverse(DenseWork& w, long long n) {
-  STM_TRY(dense_reserve(w, 0, n, kPanel));
-  STM_TRY(dense_reserve(w, 1, kPanel, n));
+  // two buffers of M's and of the panel rows' words: 64 halves per row and column each, twice
+  STM_TRY(dense_reserve(w, 0, 2 * n + 64, kPanel));
+  STM_TRY(dense_reserve(w, 1, kPanel, 2 * n + 2 * kUpCols));
   if (!grow(w.tmp, w.ntmp, n * n) || !grow(w.piv, w.npiv, n) || !grow(w.from, w.nfrom, n)) {
     set_error("coarse factorisation: out of device memory");
     return STM_ERR_OOM;
@@ -619,6 +733,9 @@ void dense_free(DenseWork& w) {
   cudaFree(w.tmp);
   cudaFree(w.piv);
   cudaFree(w.from);
+  if (w.side) cudaStreamDestroy(w.side);
+  for (cudaEvent_t e : w.ev)
+    if (e) cudaEventDestroy(e);
   w = DenseWork{};
 }
 
@@ -703,32 +820,44 @@ stm_status dense_products(const DenseWork& w, const DenseProduct* pr, int count,
   return STM_OK;
 }
 
+// Panel k + 1 needs only its own columns of update k: those come first, on s, and the other columns are updated on
+// w.side while panel k + 1 runs. Operands alternate between two buffers, since update k may still read its own
+// when panel k + 1 writes; the columns of panel k + 2 wait for update k.
 stm_status dense_inverse(DenseWork& w, double* A, int n, double* out, int* flag, cudaStream_t s) {
   if (n <= kSmallInv) {
-    if (n <= 32) STM_TRY(launch_panel<1>(A, n, 0, n, w.piv, flag, nullptr, 0, nullptr, s));
-    else if (n <= 96) STM_TRY(launch_panel<3>(A, n, 0, n, w.piv, flag, nullptr, 0, nullptr, s));
-    else STM_TRY(launch_panel<kSmallInv / 32>(A, n, 0, n, w.piv, flag, nullptr, 0, nullptr, s));
+    if (n <= 32) STM_TRY((launch_panel<1, 4>(A, n, 0, n, w.piv, flag, nullptr, nullptr, s)));
+    else if (n <= 64) STM_TRY((launch_panel<2, 8>(A, n, 0, n, w.piv, flag, nullptr, nullptr, s)));
+    else if (n <= 96) STM_TRY((launch_panel<3, kCluster>(A, n, 0, n, w.piv, flag, nullptr, nullptr, s)));
+    else STM_TRY((launch_panel<kSmallInv / 32, kCluster>(A, n, 0, n, w.piv, flag, nullptr, nullptr, s)));
   } else {
-    __half *dm = reinterpret_cast<__half*>(w.dig[0]), *dr = reinterpret_cast<__half*>(w.dig[1]);
-    const int pitch = up(n, kTileN);
-    for (int k0 = 0; k0 < n; k0 += kPanel) {
-      const int pw = std::min(kPanel, n - k0);
-      STM_TRY(launch_panel<1>(A, n, k0, pw, w.piv, flag, dm, (long long)n * kPanel, w.exps[0], s));
-      k_gj_rows<<<(pitch + 127) / 128, 128, sizeof(int) * n, s>>>(A, n, k0, pw, w.piv, flag, dr,
-                                                                  (long long)kPanel * pitch, pitch, w.exps[1]);
+    if (!w.side) STM_CUDA(cudaStreamCreateWithFlags(&w.side, cudaStreamNonBlocking));
+    for (cudaEvent_t& e : w.ev)
+      if (!e) STM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    const int pitch = up(n, kUpCols), tiles = (n + 15) / 16;
+    const long long mwords = 256LL * tiles, rwords = 16LL * pitch;
+    auto update = [&](int k0, int pw, int par, int c0, int c1, int x0, int x1, cudaStream_t st) -> stm_status {
+      uint4 *mw = (uint4*)w.dig[0] + par * mwords, *rw = (uint4*)w.dig[1] + par * rwords;
+      int *em = w.exps[0] + par * n, *er = w.exps[1] + par * n;
+      k_gj_rows<<<(c1 - c0 + 127) / 128, 128, sizeof(int) * n, st>>>(A, n, k0, pw, w.piv, c0, c1, x0, x1, flag, rw, pitch, er);
+      note_launch();
+      const int units = tiles * ((c1 - c0 + kUpCols - 1) / kUpCols);
+      k_gj_update<<<(units + 3) / 4, 128, 0, st>>>(A, n, k0, pw, mw, em, rw, er, pitch, c0, c1, x0, x1);
       note_launch();
       STM_CUDA(cudaGetLastError());
-      DenseProduct p;
-      p.a = 0;
-      p.b = 1;
-      p.m = p.n = n;
-      p.k = kPanel;
-      p.C0 = p.C = A;
-      p.ldc0 = p.ldc = n;
-      p.skip0 = k0;
-      p.skip1 = k0 + pw;
-      STM_TRY(dense_products(w, &p, 1, s));
+      return STM_OK;
+    };
+    for (int k0 = 0, k = 0; k0 < n; k0 += kPanel, ++k) {
+      const int pw = std::min(kPanel, n - k0), next = k0 + pw, nend = std::min(next + kPanel, n);
+      STM_TRY((launch_panel<1, kCluster>(A, n, k0, pw, w.piv, flag, (uint4*)w.dig[0] + (k & 1) * mwords,
+                                         w.exps[0] + (k & 1) * n, s)));
+      STM_CUDA(cudaEventRecord(w.ev[0], s));
+      if (k > 0) STM_CUDA(cudaStreamWaitEvent(s, w.ev[1], 0));  // update k - 1 is through
+      STM_CUDA(cudaStreamWaitEvent(w.side, w.ev[0], 0));
+      STM_TRY(update(k0, pw, k & 1, 0, n, next, nend, w.side));
+      STM_CUDA(cudaEventRecord(w.ev[1], w.side));
+      if (next < n) STM_TRY(update(k0, pw, k & 1, next, nend, n, n, s));
     }
+    STM_CUDA(cudaStreamWaitEvent(s, w.ev[1], 0));
   }
   k_gj_compose<<<1, 1024, 2 * sizeof(unsigned short) * n, s>>>(w.piv, n, w.from);
   note_launch();
