@@ -277,6 +277,8 @@ struct Hierarchy {
   double* cs_raw = nullptr;       // dense blocks of J_0 in slab order
   cudaStream_t chain_stream = nullptr;  // the second chain's stream
   cudaEvent_t chain_ev[2] = {};
+  double* cell_scratch = nullptr; // cell inversion: one block per resident CTA
+  long long cell_scratch_len = 0;
   int* dflag = nullptr;           // device flags: [0] singular flag, [1..2] bad cell (int64 split)
   int* dkerr = nullptr;           // device error word of the tensor-core pipelines (bounded waits)
   long long* dbad = nullptr;

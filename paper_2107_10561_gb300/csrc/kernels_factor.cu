@@ -1,178 +1,9 @@
-// Cell inverses and the coarse direct solver (FP64 arithmetic).
-//
-// Sec. 4.3: for every cell T of a level the inverse of the local Jacobian J_T is precomputed after
-// each Jacobian update. J_T holds the rows and columns of the ASSEMBLED global matrix on the
-// cell's DoFs (Sec. 4.4), gathered here straight from the CSR values through the structured
-// position map. Inversion: Gauss-Jordan elimination with partial pivoting (largest |pivot| in the
-// column, lowest row on ties) in shared memory, one CTA per cell; the result is stored
-// column-major per cell in the requested precision (FP64 / FP32 / BF16).
+// The coarse direct solver's factors (FP64; products and inverses of blocks in kernels_dense.cu).
 #include <cfloat>
 
 #include "internal.h"
 
 namespace stm {
-
-template <typename S> __device__ __forceinline__ S to_store(double v);
-template <> __device__ __forceinline__ double to_store<double>(double v) { return v; }
-template <> __device__ __forceinline__ float to_store<float>(double v) { return (float)v; }
-template <> __device__ __forceinline__ __nv_bfloat16 to_store<__nv_bfloat16>(double v) {
-  return __ushort_as_bfloat16((unsigned short)bf16_bits_rn(v));  // one rounding, straight from FP64
-}
-
-// Position in the CSR values of J_g of the entry (local row al, local col be) of cell c.
-__device__ __forceinline__ long long entry_pos(int c, int al, int be, const int* __restrict__ idx,
-                                               const int* __restrict__ cell_nodes,
-                                               const unsigned char* __restrict__ rank,
-                                               const unsigned char* __restrict__ cellrank,
-                                               const int* __restrict__ nn, const int* __restrict__ ncell,
-                                               const long long* __restrict__ rowptr, int d, int nv,
-                                               int np, int nt, int n) {
-  const int a = al / nt, ra = al - a * nt;
-  const int b = be / nt, rb = be - b * nt;
-  const long long row = idx[(long long)c * n + al];
-  const int dnv = d * nv;
-  if (ra < dnv) {
-    const int i = ra % nv;
-    const int node = cell_nodes[(long long)c * nv + i];
-    const int nni = nn[node];
-    if (rb < dnv) {
-      const int m = rb / nv, j = rb - m * nv;
-      return rowptr[row] + (long long)b * d * nni + (b > a ? np * ncell[node] : 0) + (long long)m * nni +
-             rank[((long long)c * nv + i) * nv + j];
-    }
-    if (b != a) return -1;
-    const int q = rb - dnv;
-    return rowptr[row] + (long long)a * d * nni + (long long)d * nni + (long long)cellrank[(long long)c * nv + i] * np + q;
-  }
-  if (rb >= dnv || b != a) return -1;
-  return rowptr[row] + rb;  // pressure row: columns (a, m, j) in order m * nv + j
-}
-
-// Gauss-Jordan inversion of the n x n row-major matrix A in shared memory (in place).
-// Returns false (in every thread) if a pivot is zero or not finite.
-__device__ bool gj_invert_smem(double* A, short* perm, int n, volatile int* s_piv, volatile int* s_bad) {
-  const int tid = threadIdx.x, nth = blockDim.x;
-  for (int k = 0; k < n; ++k) {
-    if (tid < 32) {
-      double best = -1.0;
-      int bi = n;
-      for (int i = k + tid; i < n; i += 32) {
-        const double v = fabs(A[i * n + k]);
-        if (v > best) { best = v; bi = i; }  // strict: the lowest row of this lane wins ties
-      }
-      for (int off = 16; off > 0; off >>= 1) {
-        const double ob = __shfl_down_sync(0xffffffffu, best, off);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (tid == 0) {
-        *s_piv = bi;
-        if (!(best > 0.0) || !(best <= DBL_MAX)) *s_bad = 1;
-        perm[k] = (short)bi;
-      }
-    }
-    __syncthreads();
-    if (*s_bad) return false;
-    const int p = *s_piv;
-    if (p != k)
-      for (int j = tid; j < n; j += nth) {
-        const double t = A[k * n + j];
-        A[k * n + j] = A[p * n + j];
-        A[p * n + j] = t;
-      }
-    __syncthreads();
-    const double pinv = 1.0 / A[k * n + k];
-    for (int j = tid; j < n; j += nth)
-      if (j != k) A[k * n + j] *= pinv;
-    __syncthreads();
-    for (int e = tid; e < n * n; e += nth) {
-      const int i = e / n, j = e - i * n;
-      if (i != k && j != k) A[e] -= A[i * n + k] * A[k * n + j];
-    }
-    __syncthreads();
-    for (int i = tid; i < n; i += nth) A[i * n + k] = (i == k) ? pinv : -A[i * n + k] * pinv;
-    __syncthreads();
-  }
-  // undo the row interchanges as column interchanges, last first
-  for (int k = n - 1; k >= 0; --k) {
-    const int p = perm[k];
-    if (p != k)
-      for (int i = tid; i < n; i += nth) {
-        const double t = A[i * n + k];
-        A[i * n + k] = A[i * n + p];
-        A[i * n + p] = t;
-      }
-    __syncthreads();
-  }
-  return true;
-}
-
-template <typename S>
-__global__ void __launch_bounds__(512) k_cell_inverse(
-    const int* __restrict__ idx, const int* __restrict__ cell_nodes, const unsigned char* __restrict__ rank,
-    const unsigned char* __restrict__ cellrank, const int* __restrict__ nn, const int* __restrict__ ncell,
-    const long long* __restrict__ rowptr, const double* __restrict__ val, S* __restrict__ inv, int C, int d,
-    int nv, int np, int nt, int n, int ld, int* flag, long long* bad) {
-  extern __shared__ double sm[];
-  double* A = sm;
-  short* perm = reinterpret_cast<short*>(A + (size_t)n * n);
-  __shared__ int s_piv, s_bad;
-  for (int c = blockIdx.x; c < C; c += gridDim.x) {
-    if (threadIdx.x == 0) s_bad = 0;
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-      const int al = e / n, be = e - al * n;
-      const long long pos = entry_pos(c, al, be, idx, cell_nodes, rank, cellrank, nn, ncell, rowptr, d, nv, np, nt, n);
-      A[e] = pos >= 0 ? val[pos] : 0.0;
-    }
-    __syncthreads();
-    const bool ok = gj_invert_smem(A, perm, n, &s_piv, &s_bad);
-    if (!ok) {
-      if (threadIdx.x == 0 && atomicCAS(flag, 0, 1) == 0) *bad = c;
-      __syncthreads();
-      continue;
-    }
-    S* out = inv + (size_t)c * n * ld;
-    for (int e = threadIdx.x; e < n * ld; e += blockDim.x) {
-      const int j = e / ld, i = e - j * ld;  // column-major store: element (i, j) at j * ld + i
-      out[e] = to_store<S>(i < n ? A[i * n + j] : 0.0);
-    }
-    __syncthreads();
-  }
-}
-
-static size_t storage_bytes(int prec) { return prec == STM_F64 ? 8 : prec == STM_F32 ? 4 : 2; }
-
-stm_status factor_level(Hierarchy& H, int g, cudaStream_t s) {
-  Level& L = H.L[g];
-  const size_t nn2 = (size_t)L.n * L.n;
-  const InvLayout lay = inv_layout(L.n, H.p.inv_precision);
-  if (!L.inv) STM_CUDA(cudaMalloc(&L.inv, storage_bytes(H.p.inv_precision) * (size_t)L.n * lay.ld * L.C));
-  const size_t smem = sizeof(double) * nn2 + sizeof(short) * L.n + 16;
-  int dev = 0, maxsm = 0;
-  STM_CUDA(cudaGetDevice(&dev));
-  STM_CUDA(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (smem + 64 > (size_t)maxsm) {
-    set_error("factor_cells: cell matrix does not fit in shared memory");
-    return STM_ERR_INVALID_ARG;
-  }
-  const int threads = L.n >= 128 ? 512 : 256;
-  int sms = 0;
-  STM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int blocks = std::min(L.C, sms * 16);
-#define LAUNCH_INV(T)                                                                                  \
-  do {                                                                                                \
-    STM_CUDA(cudaFuncSetAttribute(k_cell_inverse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-    k_cell_inverse<T><<<blocks, threads, smem, s>>>(L.idx, L.cell_nodes, L.rank, L.cellrank, L.nn, L.ncell,  \
-                                                    L.rowptr, L.val, (T*)L.inv, L.C, L.dim, L.nv, L.np,     \
-                                                    L.nt, L.n, lay.ld, H.dflag, H.dbad); note_launch();                            \
-  } while (0)
-  if (H.p.inv_precision == STM_F64) LAUNCH_INV(double);
-  else if (H.p.inv_precision == STM_F32) LAUNCH_INV(float);
-  else LAUNCH_INV(__nv_bfloat16);
-#undef LAUNCH_INV
-  STM_CUDA(cudaGetLastError());
-  return STM_OK;
-}
 
 // ---------------------------------------------------------------------------------------------
 // Coarse level: explicit FP64 inverse of J_0 by Gauss-Jordan with partial pivoting in global memory
