@@ -264,15 +264,17 @@ struct Hierarchy {
   long long N0 = 0;
   double* cinvT = nullptr;  // [N0][N0] its transpose, row-major (the adjoint coarse solve reads rows too)
   // coarse solve through the twisted block factors in x-slab order (large coarse levels; cinv is then
-  // not formed): cs_nx slabs eliminated from both ends towards slab cs_t, row offsets cs_off [nx + 1],
-  // block offsets cs_pos [8][nx] into cs_store (inverse, lower and upper chain blocks, back-substitution
-  // block, for J_0 and for J_0^T), slab of every permuted row, permuted position of every row; work
-  // vectors for one column and for 32 interleaved columns
+  // not formed): cs_nx slabs of at most cs_maxnb rows eliminated from both ends towards slab cs_t, row
+  // offsets cs_off [nx + 1], the blocks in cs_store (inverse, lower and upper chain blocks, back-
+  // substitution block, for J_0 and for J_0^T) and their digits in cs_words with the powers of two in
+  // cs_exps (offsets of both per kind and slab in cs_wpos [2][8][nx]), permuted position of every row;
+  // work vectors for one column and for 32 interleaved columns, the latter's partial sums
   bool coarse_slab = false;
-  int cs_nx = 0, cs_t = 0;
-  long long *cs_off = nullptr, *cs_pos = nullptr;
-  int *cs_rowslab = nullptr, *cs_perm = nullptr;
-  double *cs_store = nullptr, *cs_u = nullptr, *cs_v = nullptr, *cs_mu = nullptr, *cs_mv = nullptr;
+  int cs_nx = 0, cs_t = 0, cs_maxnb = 0;
+  long long *cs_off = nullptr, *cs_wpos = nullptr;
+  int *cs_perm = nullptr, *cs_exps = nullptr;
+  void* cs_words = nullptr;
+  double *cs_store = nullptr, *cs_u = nullptr, *cs_v = nullptr, *cs_mu = nullptr, *cs_mv = nullptr, *cs_part = nullptr;
   DenseWork dw[2];                // coarse factorisation: one work space per elimination chain
   double* cs_raw = nullptr;       // dense blocks of J_0 in slab order
   cudaStream_t chain_stream = nullptr;  // the second chain's stream
@@ -410,7 +412,10 @@ stm_status smoother_defect(Hierarchy& H, int g, const double* x, const double* b
 stm_status vanka_step(Hierarchy& H, int g, const double* r, double* d, int transpose,
                       bool d_is_zero, cudaStream_t s, bool d32_current = false);
 stm_status coarse_apply(Hierarchy& H, const double* r, double* d, int transpose, cudaStream_t s);
-// the coarse solve through the slab block-LU factors (kernels_coarse.cu): one column, or 32 interleaved
+// the coarse solve through the slab block-LU factors (kernels_coarse.cu): their digits, built with the
+// factors; one column, or 32 interleaved
+stm_status coarse_slab_words(Hierarchy& H, const std::vector<long long>& off, const std::vector<long long>& cpos,
+                             cudaStream_t s);
 stm_status coarse_slab_apply(Hierarchy& H, const double* r, double* d, int transpose, cudaStream_t s);
 stm_status coarse_slab_apply_multi(Hierarchy& H, const double* R, double* D, cudaStream_t s);
 // wnod: nodal linearisation velocity [K][d][R] of the finest level to use instead of the stored one

@@ -246,10 +246,10 @@ static stm_status invert_block(DenseWork& w, double* M, long long nb, double* ou
 // of the one-sided block LU. The Schur complements of J_0^T in the same order are the S_b^T, so the
 // transposed system needs no inversion of its own: its blocks are S_b^{-T}, (A_{b-1,b} S_b^{-1})^T (lower
 // chain, or back-substitution below the twist) and (A_{b+1,b} S_b^{-1})^T (upper chain, or back-
-// substitution above the twist). Every block is kept row-major in H.cs_store at H.cs_pos[kind][b], kinds
+// substitution above the twist). Every block is kept row-major in H.cs_store at cpos[kind][b], kinds
 // 0..3 (inverse, lower chain G, upper chain G', back-substitution W or V) for J_0 and 4..7 for J_0^T.
 static stm_status twisted_slab_factors(Hierarchy& H, const Level& L, const std::vector<long long>& off,
-                                       const std::vector<int>& iperm, const std::vector<int>& blk, double* raw,
+                                       const std::vector<int>& iperm, double* raw,
                                        const std::vector<long long>& dpos, const std::vector<long long>& lpos,
                                        const std::vector<long long>& upos, double* scal, cudaStream_t s) {
   enum { K_INV = 0, K_LO = 1, K_UP = 2, K_BACK = 3, K_T = 4 };
@@ -273,8 +273,7 @@ static stm_status twisted_slab_factors(Hierarchy& H, const Level& L, const std::
   if ((!H.cs_store && cudaMalloc(&H.cs_store, sizeof(double) * ct)) ||
       (!H.cs_u && cudaMalloc(&H.cs_u, sizeof(double) * n)) || (!H.cs_v && cudaMalloc(&H.cs_v, sizeof(double) * n)) ||
       (!H.cs_off && cudaMalloc(&H.cs_off, sizeof(long long) * (nx + 1))) ||
-      (!H.cs_pos && cudaMalloc(&H.cs_pos, sizeof(long long) * 8 * nx)) ||
-      (!H.cs_rowslab && cudaMalloc(&H.cs_rowslab, sizeof(int) * n)) || (!H.cs_perm && cudaMalloc(&H.cs_perm, sizeof(int) * n))) {
+      (!H.cs_perm && cudaMalloc(&H.cs_perm, sizeof(int) * n))) {
     cudaGetLastError();
     set_error("coarse factorisation: out of device memory");
     return STM_ERR_OOM;
@@ -368,16 +367,16 @@ static stm_status twisted_slab_factors(Hierarchy& H, const Level& L, const std::
   }
   std::vector<long long> hoff(off.begin(), off.begin() + nx + 1);
   cudaMemcpyAsync(H.cs_off, hoff.data(), sizeof(long long) * (nx + 1), cudaMemcpyHostToDevice, s);
-  cudaMemcpyAsync(H.cs_pos, cpos.data(), sizeof(long long) * 8 * nx, cudaMemcpyHostToDevice, s);
-  cudaMemcpyAsync(H.cs_rowslab, blk.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s);
   cudaMemcpyAsync(H.cs_perm, iperm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s);
+  H.cs_nx = nx;
+  H.cs_t = t;
+  H.cs_maxnb = (int)maxnb;
+  STM_TRY(coarse_slab_words(H, off, cpos, s));
   const cudaError_t e1 = cudaGetLastError(), e2 = cudaStreamSynchronize(s);
   if (e1 != cudaSuccess || e2 != cudaSuccess) {
     set_error("coarse factorisation: CUDA error");
     return STM_ERR_CUDA;
   }
-  H.cs_nx = nx;
-  H.cs_t = t;
   H.coarse_slab = true;
   return STM_OK;
 }
@@ -450,7 +449,7 @@ stm_status factor_coarse(Hierarchy& H, cudaStream_t s) {
                                                                           H.dflag + 1);
     note_launch();
     if (use_slab) {
-      st = twisted_slab_factors(H, L, off, iperm, blk, store, dpos, lpos, upos, scal, s);
+      st = twisted_slab_factors(H, L, off, iperm, store, dpos, lpos, upos, scal, s);
       break;
     }
     // C (m x n) = [C0] + alpha A B, ld of each as given
