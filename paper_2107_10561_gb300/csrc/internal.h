@@ -250,6 +250,7 @@ struct DenseWork {
   double* tmp = nullptr;
   int *piv = nullptr, *from = nullptr;
   long long ntmp = 0, npiv = 0, nfrom = 0;
+  bool overlap = false;           // dense_inverse may use a stream of its own beside the caller's
   cudaStream_t side = nullptr;    // updates of the columns that the next panel does not need
   cudaEvent_t ev[2] = {};
 };

@@ -822,7 +822,11 @@ stm_status dense_products(const DenseWork& w, const DenseProduct* pr, int count,
 
 // Panel k + 1 needs only its own columns of update k: those come first, on s, and the other columns are updated on
 // w.side while panel k + 1 runs. Operands alternate between two buffers, since update k may still read its own
-// when panel k + 1 writes; the columns of panel k + 2 wait for update k.
+// when panel k + 1 writes; the columns of panel k + 2 wait for update k. Where the caller allows no second stream
+// (w.overlap) all of it runs on s: once two streams have run in a context, every launch after that costs a little
+// more, for good (a 2D adjoint solve of 13 iterations: 5.43 -> 5.68 ms), and one update of all columns costs a 2D
+// Newton step no more than two side by side (58.1 against 59.5 ms). The slab chains of 3D use two streams anyway
+// (dG(0) step: 43.5 -> 39.1 ms with the overlap).
 stm_status dense_inverse(DenseWork& w, double* A, int n, double* out, int* flag, cudaStream_t s) {
   if (n <= kSmallInv) {
     if (n <= 32) STM_TRY((launch_panel<1, 4>(A, n, 0, n, w.piv, flag, nullptr, nullptr, s)));
@@ -830,9 +834,11 @@ stm_status dense_inverse(DenseWork& w, double* A, int n, double* out, int* flag,
     else if (n <= 96) STM_TRY((launch_panel<3, kCluster>(A, n, 0, n, w.piv, flag, nullptr, nullptr, s)));
     else STM_TRY((launch_panel<kSmallInv / 32, kCluster>(A, n, 0, n, w.piv, flag, nullptr, nullptr, s)));
   } else {
-    if (!w.side) STM_CUDA(cudaStreamCreateWithFlags(&w.side, cudaStreamNonBlocking));
-    for (cudaEvent_t& e : w.ev)
-      if (!e) STM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    if (w.overlap) {
+      if (!w.side) STM_CUDA(cudaStreamCreateWithFlags(&w.side, cudaStreamNonBlocking));
+      for (cudaEvent_t& e : w.ev)
+        if (!e) STM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    }
     const int pitch = up(n, kUpCols), tiles = (n + 15) / 16;
     const long long mwords = 256LL * tiles, rwords = 16LL * pitch;
     auto update = [&](int k0, int pw, int par, int c0, int c1, int x0, int x1, cudaStream_t st) -> stm_status {
@@ -848,16 +854,20 @@ stm_status dense_inverse(DenseWork& w, double* A, int n, double* out, int* flag,
     };
     for (int k0 = 0, k = 0; k0 < n; k0 += kPanel, ++k) {
       const int pw = std::min(kPanel, n - k0), next = k0 + pw, nend = std::min(next + kPanel, n);
-      STM_TRY((launch_panel<1, kCluster>(A, n, k0, pw, w.piv, flag, (uint4*)w.dig[0] + (k & 1) * mwords,
-                                         w.exps[0] + (k & 1) * n, s)));
+      const int par = w.overlap ? k & 1 : 0;
+      STM_TRY((launch_panel<1, kCluster>(A, n, k0, pw, w.piv, flag, (uint4*)w.dig[0] + par * mwords, w.exps[0] + par * n, s)));
+      if (!w.overlap) {
+        STM_TRY(update(k0, pw, par, 0, n, n, n, s));
+        continue;
+      }
       STM_CUDA(cudaEventRecord(w.ev[0], s));
       if (k > 0) STM_CUDA(cudaStreamWaitEvent(s, w.ev[1], 0));  // update k - 1 is through
       STM_CUDA(cudaStreamWaitEvent(w.side, w.ev[0], 0));
-      STM_TRY(update(k0, pw, k & 1, 0, n, next, nend, w.side));
+      STM_TRY(update(k0, pw, par, 0, n, next, nend, w.side));
       STM_CUDA(cudaEventRecord(w.ev[1], w.side));
-      if (next < n) STM_TRY(update(k0, pw, k & 1, next, nend, n, n, s));
+      if (next < n) STM_TRY(update(k0, pw, par, next, nend, n, n, s));
     }
-    STM_CUDA(cudaStreamWaitEvent(s, w.ev[1], 0));
+    if (w.overlap) STM_CUDA(cudaStreamWaitEvent(s, w.ev[1], 0));
   }
   k_gj_compose<<<1, 1024, 2 * sizeof(unsigned short) * n, s>>>(w.piv, n, w.from);
   note_launch();

@@ -345,6 +345,7 @@ static stm_status twisted_slab_factors(Hierarchy& H, const Level& L, const std::
   long long maxnb = 0;
   for (int b = 0; b < nx; ++b) maxnb = std::max(maxnb, rows(b));
   for (DenseWork& w : H.dw) {
+    w.overlap = true;
     STM_TRY(dense_reserve_inverse(w, maxnb));
     for (int q = 0; q < DenseWork::kSlots; ++q) STM_TRY(dense_reserve(w, q, maxnb, maxnb));
   }
