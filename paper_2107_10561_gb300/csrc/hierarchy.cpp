@@ -493,8 +493,21 @@ static stm_status build_level(const stm_params& p, int g, Level& L, std::vector<
   STM_TRY(upload(&L.nbase, nbase));
   STM_CUDA(cudaMalloc((void**)&L.spmv_work, sizeof(unsigned) * 2));
   STM_CUDA(cudaMemset(L.spmv_work, 0, sizeof(unsigned) * 2));
-  STM_CUDA(cudaMalloc((void**)&L.nval, sizeof(double) * nbase[R]));
-  L.nval_len = nbase[R];
+  L.nval_len = L.nval_cap = nbase[R];
+  L.limb_lanes = limb_lanes(L);
+  if (L.limb_lanes) {
+    // runs of limb_lanes neighbours and pressures, the last one of a node padded
+    const int vl = L.limb_lanes;
+    auto up = [vl](long long v) { return (v + vl - 1) / vl * vl; };
+    std::vector<long long> lbase(R + 1, 0);
+    for (int nd = 0; nd < R; ++nd)
+      lbase[nd + 1] = lbase[nd] + (long long)(L.K * d) * (L.K * d * up(nn[nd]) + up((long long)np * ncell[nd]));
+    L.nval_cap = lbase[R];
+    STM_TRY(upload(&L.lbase, lbase));
+    STM_CUDA(cudaMalloc((void**)&L.nexp, sizeof(int) * (size_t)R * (L.K * d + 1)));
+    STM_CUDA(cudaMalloc((void**)&L.cexp, sizeof(int2) * C));
+  }
+  STM_CUDA(cudaMalloc((void**)&L.nval, sizeof(double) * L.nval_cap));
   {
     const long long prows = ((long long)L.K * C * np + 31) / 32 * 32;
     L.pval_len = prows * d * L.nv;
@@ -772,7 +785,7 @@ void free_hierarchy(Hierarchy& H) {
   for (Level& L : H.L) {
     void* ptrs[] = {L.idx, L.cell_nodes, L.cell_xyz, L.bmask, L.rank, L.cellrank, L.nn, L.ncell, L.rowptr, L.nbr_ptr, L.nbr,
                     L.node_cells, L.job_nodes, L.nbase, L.spmv_work, L.nval, L.pvalT, L.nvalJT, L.pvalJT, L.nval32, L.pval32,
-                    L.nvalJT32, L.pvalJT32, L.x32,
+                    L.nvalJT32, L.pvalJT32, L.x32, L.nexp, L.nexpJT, L.cexp, L.lbase,
                     L.colidx, L.val, L.valT, L.ref, L.inj, L.wnod, L.inv, L.wmult, L.own_ptr,
                     L.own_pos, L.last_owner, L.colour_cells, L.colour_jobs, L.Y, L.P_rowptr, L.P_col, L.P_val,
                     L.Rt_rowptr, L.Rt_col, L.Rt_val, L.tv_ptr, L.tv_node, L.tv_w, L.tc_ptr, L.tc_node,

@@ -182,12 +182,19 @@ struct Level {
   // t = m*nv + j of row pr at pvalT[((pr/32)*d*nv + t)*32 + pr%32] (rows padded to a multiple of 32)
   double* pvalT = nullptr;
   double *nvalJT = nullptr, *pvalJT = nullptr;  // the same two copies for J^T (built with valT)
+  // limb_lanes > 0: nval and nvalJT hold two-limb integers instead (limbs.h), positions in runs of limb_lanes;
+  // per node the K*d row exponents and the offset of the pressure columns; cexp: per cell, x's exponents
+  int limb_lanes = 0;
+  long long* lbase = nullptr;              // [R+1] start of each node, in values
+  int *nexp = nullptr, *nexpJT = nullptr;  // [R][K*d + 1]
+  int2* cexp = nullptr;                    // [C]
   unsigned* spmv_work = nullptr;  // [2] unit counter and finished-CTA count of the FP64 product (zeroed)
   // FP32 copies of nval/pvalT (and of nvalJT/pvalJT) in the same layout, for the V-cycle's defects
   // r - J_g d with defect_precision = STM_F32; null otherwise
   float *nval32 = nullptr, *pval32 = nullptr, *nvalJT32 = nullptr, *pvalJT32 = nullptr;
   float* x32 = nullptr;  // [N] the defect's d rounded to FP32
-  long long nval_len = 0, pval_len = 0;          // entries of nval and pvalT
+  long long nval_len = 0, pval_len = 0;          // entries of the node blocks and of pvalT
+  long long nval_cap = 0;                        // entries allocated for nval and nvalJT
   int* ncell = nullptr;           // [R] number of cells containing the node
   long long* rowptr = nullptr;    // [N+1]
   int* colidx = nullptr;          // [nnz]
@@ -385,12 +392,17 @@ stm_status transfer_restrict(const Level& F, const Level& Cl, const double* fine
 // fine += P coarse; with fine32 non-null the updated entries are also stored rounded to FP32 there
 stm_status transfer_prolong_add(const Level& F, const Level& Cl, const double* coarse, double* fine, cudaStream_t s,
                                 float* fine32 = nullptr);
-stm_status spmv_nodeblock(const Level& L, const double* nval, const double* pvalT, const double* x, const double* b,
-                          double* y, int mode, cudaStream_t s,
-                          const int* jobs = nullptr, int njobs = -1);
-stm_status build_nodeblock(Level& L, cudaStream_t s);
-// node-block and warp-transposed pressure-row copies of any value array on J's pattern (J or J^T)
-stm_status build_nodeblock_from(const Level& L, const double* val, double* nval, double* pvalT, cudaStream_t s);
+stm_status spmv_nodeblock(const Level& L, int transpose, const double* x, const double* b, double* y, int mode,
+                          cudaStream_t s, const int* jobs = nullptr, int njobs = -1);
+// lanes per node in the FP64 product, and the same where the level keeps limbs (0: FP64 values)
+int node_lanes(const Level& L);
+int limb_lanes(const Level& L);
+// the same product of the levels that keep limbs, and their copy of the velocity rows (kernels_limb_spmv.cu)
+stm_status spmv_limbs(const Level& L, int transpose, const double* x, const double* b, double* y, int mode,
+                      cudaStream_t s, const int* jobs, int njobs);
+stm_status build_limbs(const Level& L, const double* val, double* nval, int* nexp, cudaStream_t s);
+// node-block and warp-transposed pressure-row copies of J's or J^T's values
+stm_status build_nodeblock(const Level& L, int transpose, cudaStream_t s);
 // y = b - J_g x (transpose: J_g^T) over the FP32 copies of the values: x rounded to FP32 into L.x32
 // (skipped when x32_current: the kernel that last wrote x stored it there rounded), FP32 products
 // and sums, b and y in FP64

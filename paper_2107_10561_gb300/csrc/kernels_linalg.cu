@@ -109,10 +109,11 @@ stm_status ensure_transpose(Hierarchy& H, int g, cudaStream_t s) {
     return STM_ERR_STATE;
   }
   // node-block and pressure-row copies of J^T for the transposed SpMV
-  STM_CUDA(cudaMalloc(&L.nvalJT, sizeof(double) * L.nval_len));
+  STM_CUDA(cudaMalloc(&L.nvalJT, sizeof(double) * L.nval_cap));
   STM_CUDA(cudaMalloc(&L.pvalJT, sizeof(double) * L.pval_len));
   STM_CUDA(cudaMemsetAsync(L.pvalJT, 0, sizeof(double) * L.pval_len, s));
-  STM_TRY(build_nodeblock_from(L, L.valT, L.nvalJT, L.pvalJT, s));
+  if (L.limb_lanes) STM_CUDA(cudaMalloc(&L.nexpJT, sizeof(int) * L.R * (L.K * L.dim + 1)));
+  STM_TRY(build_nodeblock(L, 1, s));
   if (H.p.defect_precision == STM_F32) STM_TRY(build_values_f32(L, 1, s));
   return STM_OK;
 }
@@ -122,8 +123,7 @@ stm_status jacobian_apply(Hierarchy& H, int g, const double* x, const double* b,
   Level& L = H.L[g];
   if (transpose) STM_TRY(ensure_transpose(H, g, s));
   ProfScope ps(&H, STM_KCLASS_JACOBIAN_SPMV, s, 8.0 * (double)L.nnz + 24.0 * (double)L.N, g);
-  if (!transpose) return spmv_nodeblock(L, L.nval, L.pvalT, x, b, y, mode, s);
-  return spmv_nodeblock(L, L.nvalJT, L.pvalJT, x, b, y, mode, s);
+  return spmv_nodeblock(L, transpose, x, b, y, mode, s);
 }
 
 stm_status jacobian_defect_colour(Hierarchy& H, int g, int colour, const double* x, const double* b, double* y,
@@ -132,8 +132,7 @@ stm_status jacobian_defect_colour(Hierarchy& H, int g, int colour, const double*
   if (transpose) STM_TRY(ensure_transpose(H, g, s));
   const int j0 = L.colour_job_off[colour], nj = L.colour_job_off[colour + 1] - j0;
   ProfScope ps(&H, STM_KCLASS_JACOBIAN_SPMV, s, 8.0 * (double)L.nnz * nj / std::max(L.R, 1) + 24.0 * (double)L.N, g);
-  return spmv_nodeblock(L, transpose ? L.nvalJT : L.nval, transpose ? L.pvalJT : L.pvalT, x, b, y, 1, s,
-                        L.colour_jobs + j0, nj);
+  return spmv_nodeblock(L, transpose, x, b, y, 1, s, L.colour_jobs + j0, nj);
 }
 
 // The outer solver is flexible GMRES (Sec. 3): it keeps every preconditioned vector z_j = V(v_j), so

@@ -16,7 +16,8 @@
 //   - warp-transposed pressure rows: one lane per row, entry t of 32 consecutive rows contiguous.
 // Column indices are never read. In FP64, issue slots of the FP64 pipe are the limit (one FP64 warp
 // instruction every 16 cycles per SM); results equal the plain CSR product up to FP64 summation
-// order. In FP32 the arithmetic is cheap and the loads in flight per SM set the pace.
+// order. FP64 values are kept on 2D levels only, and there where limb_lanes() says so: the others' velocity
+// rows are integers (kernels_limb_spmv.cu). In FP32 the arithmetic is cheap and the loads in flight per SM set the pace.
 #include "internal.h"
 
 namespace stm {
@@ -74,9 +75,10 @@ __device__ __forceinline__ int scatter_index(int lane, int* writer_mask) {
 //   pos < (a+1) d nn                 : p = pos                        (velocity blocks b <= a)
 //   next n_p nc entries (pressure)   : p = K d nn + (pos - (a+1) d nn)
 //   beyond                           : p = pos - n_p nc               (velocity blocks b > a)
+template <typename T>
 __global__ void k_build_nodeblock(const long long* __restrict__ rowptr, const double* __restrict__ val,
                                   const int* __restrict__ nbr_ptr, const int* __restrict__ ncell,
-                                  const long long* __restrict__ nbase, double* __restrict__ nval, long long block,
+                                  const long long* __restrict__ nbase, T* __restrict__ nval, long long block,
                                   int R, int K, int D, int NP) {
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -94,7 +96,7 @@ __global__ void k_build_nodeblock(const long long* __restrict__ rowptr, const do
           if (pos < lim) p = pos;
           else if (pos < lim + NP * nc) p = KD * nn + (pos - lim);
           else p = pos - NP * nc;
-          nval[nbase[i] + (long long)p * KD + a * D + l] = val[rb + pos];
+          nval[nbase[i] + (long long)p * KD + a * D + l] = (T)val[rb + pos];
         }
       }
   }
@@ -116,14 +118,21 @@ __global__ void k_build_pval(const long long* __restrict__ rowptr, const double*
   }
 }
 
-stm_status build_nodeblock(Level& L, cudaStream_t s) { return build_nodeblock_from(L, L.val, L.nval, L.pvalT, s); }
-
-stm_status build_nodeblock_from(const Level& L, const double* val, double* nval, double* pvalT, cudaStream_t s) {
+template <typename T>
+static stm_status build_velocity(const Level& L, const double* val, T* nval, cudaStream_t s) {
   const int blocks = (int)std::min<long long>(((long long)L.R * 32 + 255) / 256, sm_count() * 8LL);
   k_build_nodeblock<<<blocks, 256, 0, s>>>(L.rowptr, val, L.nbr_ptr, L.ncell, L.nbase, nval, L.block, L.R, L.K,
                                            L.dim, L.np);
   note_launch();
   STM_CUDA(cudaGetLastError());
+  return STM_OK;
+}
+
+stm_status build_nodeblock(const Level& L, int transpose, cudaStream_t s) {
+  const double* val = transpose ? L.valT : L.val;
+  double *nval = transpose ? L.nvalJT : L.nval, *pvalT = transpose ? L.pvalJT : L.pvalT;
+  if (L.limb_lanes) STM_TRY(build_limbs(L, val, nval, transpose ? L.nexpJT : L.nexp, s));
+  else STM_TRY(build_velocity(L, val, nval, s));
   const long long npr = (long long)L.K * L.C * L.np;
   const int pblocks = (int)std::min<long long>((npr + 255) / 256, sm_count() * 8LL);
   k_build_pval<<<std::max(pblocks, 1), 256, 0, s>>>(L.rowptr, val, pvalT, L.block, L.R, L.C, L.K, L.dim, L.np,
@@ -369,8 +378,8 @@ __global__ void __launch_bounds__(256) k_spmv_nb_dyn(
         const double* blk = nval + nbase[i];
         const int npv = KD * nn;
         // U positions per step: the loads of all U are issued before the first FMA waits (U = 1 is used:
-        // two positions per step measured 93.2 against 89.4 us on the finest 2D dG(2) level and 567
-        // against 564 us on the finest 3D dG(1) level, with fewer resident warps at 64-80 registers)
+        // two positions per step measured 93.2 against 89.4 us on 536,448 unknowns of 2D dG(2), with
+        // fewer resident warps at 64-80 registers)
         int jk[U], bk[U];
         jk[0] = lane;
         bk[0] = 0;
@@ -555,36 +564,32 @@ static stm_status launch_nb_dyn(const Level& L, const double* nval, const double
   return STM_OK;
 }
 
-stm_status spmv_nodeblock(const Level& L, const double* nval, const double* pvalT, const double* x, const double* b,
-                          double* y, int mode, cudaStream_t s, const int* jobs, int njobs) {
+// lanes per node as for the static product: short groups on large levels, 16 / 32 on small ones
+int node_lanes(const Level& L) {
+  const long long per_sm_threads = 1024;
+  if ((long long)L.R * 16 < (long long)sms_count() * per_sm_threads / 4) return 32;
+  if ((long long)L.R * (L.dim == 2 ? 4 : 8) < (long long)sms_count() * per_sm_threads) return 16;
+  return L.dim == 2 ? 4 : 8;
+}
+
+stm_status spmv_nodeblock(const Level& L, int transpose, const double* x, const double* b, double* y, int mode,
+                          cudaStream_t s, const int* jobs, int njobs) {
+  if (L.limb_lanes) return spmv_limbs(L, transpose, x, b, y, mode, s, jobs, njobs);
+  const double *nval = transpose ? L.nvalJT : L.nval, *pvalT = transpose ? L.pvalJT : L.pvalT;
   if (!jobs) {
     jobs = L.job_nodes;
     njobs = L.R;
   }
-  // lanes per node as for the static product: short groups on large levels, 16 / 32 on small ones
-  const long long per_sm_threads = 1024;
-  int cls = 0;
-  if ((long long)L.R * (L.dim == 2 ? 4 : 8) < (long long)sms_count() * per_sm_threads) cls = 100;
-  if ((long long)L.R * 16 < (long long)sms_count() * per_sm_threads / 4) cls = 200;
+  const int vl = node_lanes(L), cls = vl == 32 ? 200 : vl == 16 ? 100 : 0;
   switch (L.dim * 10 + L.K + cls) {
     case 21: return launch_nb_dyn<4, 1, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
     case 22: return launch_nb_dyn<4, 2, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
-    case 23: return launch_nb_dyn<4, 3, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
-    case 31: return launch_nb_dyn<8, 1, 3, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
-    case 32: return launch_nb_dyn<8, 2, 3, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
-    case 33: return launch_nb_dyn<8, 3, 3, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
     case 121: return launch_nb_dyn<16, 1, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
     case 122: return launch_nb_dyn<16, 2, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
     case 123: return launch_nb_dyn<16, 3, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
-    case 131: return launch_nb_dyn<16, 1, 3, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
-    case 132: return launch_nb_dyn<16, 2, 3, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
-    case 133: return launch_nb_dyn<16, 3, 3, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
     case 221: return launch_nb_dyn<32, 1, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
     case 222: return launch_nb_dyn<32, 2, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
     case 223: return launch_nb_dyn<32, 3, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
-    case 231: return launch_nb_dyn<32, 1, 3, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
-    case 232: return launch_nb_dyn<32, 2, 3, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
-    case 233: return launch_nb_dyn<32, 3, 3, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
     default:
       set_error("node-block SpMV: unsupported (dim, k)");
       return STM_ERR_INVALID_ARG;
@@ -618,7 +623,7 @@ stm_status build_values_f32(Level& L, int transpose, cudaStream_t s) {
   if (!n32) STM_CUDA(cudaMalloc((void**)&n32, sizeof(float) * std::max<long long>(1, L.nval_len)));
   if (!p32) STM_CUDA(cudaMalloc((void**)&p32, sizeof(float) * std::max<long long>(1, L.pval_len)));
   if (!L.x32) STM_CUDA(cudaMalloc((void**)&L.x32, sizeof(float) * std::max<long long>(1, L.N)));
-  STM_TRY(round_f32(nv, n32, L.nval_len, s));
+  STM_TRY(build_velocity(L, transpose ? L.valT : L.val, n32, s));
   if (pv) STM_TRY(round_f32(pv, p32, L.pval_len, s));
   return STM_OK;
 }
