@@ -430,7 +430,9 @@ stm_status factor_level(Hierarchy& H, int g, cudaStream_t s) {
   }
   const size_t smem = cell_smem(n, in_smem).total;
   a.scratch = in_smem ? nullptr : H.cell_scratch;
-  return per_sm == 4 ? launch<128>(H, a, L.inv, blocks, smem, s) : launch<256>(H, a, L.inv, blocks, smem, s);
+  if (per_sm == 4) STM_TRY(launch<128>(H, a, L.inv, blocks, smem, s));
+  else STM_TRY(launch<256>(H, a, L.inv, blocks, smem, s));
+  return H.p.inv_precision == STM_F64 ? inverse_limbs(L, s) : STM_OK;
 }
 
 }  // namespace stm
