@@ -309,59 +309,75 @@ stm_status vec_scale_to(double* y, const double* x, const double* sc, int inv, l
 }
 
 // part[v][blk] = partial sum of V[v] . w over the block's chunk; then out[v] = sum_blk part (fixed order)
-// Four dot products per pass over w (w read once for each group of four); per product the same
-// reduction tree as a single one: warp shuffles, then the warp sums in warp order.
-__global__ void k_dots_partial(const double* __restrict__ V, int nv, const double* __restrict__ w, long long n,
-                               double* __restrict__ part) {
+// Four dot products per block (w read once for the four); blockIdx.y walks the groups of four, side by side: in
+// short solves the FP64 sums are the time (74 clocks per warp and sum, 4 warps per sub-core), so neither the groups
+// nor the four warp sums of a group follow one another (warp u joins product u), and a warp sums as few as it can.
+__global__ void __launch_bounds__(256) k_dots_partial(const double* __restrict__ V, int nv, const double* __restrict__ w,
+                                                      long long n, double* __restrict__ part) {
   constexpr int CH = 4;
-  __shared__ double red[CH][32];
-  for (int v0 = 0; v0 < nv; v0 += CH) {
-    const int nc = min(CH, nv - v0);
-    double s[CH];
+  __shared__ double red[CH][8];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int v0 = blockIdx.y * CH, nc = min(CH, nv - v0), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double s[CH];
 #pragma unroll
-    for (int u = 0; u < CH; ++u) s[u] = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-      const double wi = w[i];
+  for (int u = 0; u < CH; ++u) s[u] = 0.0;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const double wi = w[i];
 #pragma unroll
-      for (int u = 0; u < CH; ++u)
-        if (u < nc) s[u] += V[(long long)(v0 + u) * n + i] * wi;
-    }
+    for (int u = 0; u < CH; ++u)
+      if (u < nc) s[u] += V[(long long)(v0 + u) * n + i] * wi;
+  }
+  // halves of the products change places first, so that a warp adds 6 times instead of 20
+  const bool up = lane & 16, odd = lane & 8;
+  double p0 = up ? s[2] : s[0], p1 = up ? s[3] : s[1];
+  p0 += __shfl_xor_sync(0xffffffffu, up ? s[0] : s[2], 16);
+  p1 += __shfl_xor_sync(0xffffffffu, up ? s[1] : s[3], 16);
+  double p = odd ? p1 : p0;
+  p += __shfl_xor_sync(0xffffffffu, odd ? p0 : p1, 8);
 #pragma unroll
-    for (int u = 0; u < CH; ++u) {
-      for (int off = 16; off > 0; off >>= 1) s[u] += __shfl_down_sync(0xffffffffu, s[u], off);
-      if ((threadIdx.x & 31) == 0) red[u][threadIdx.x >> 5] = s[u];
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      for (int u = 0; u < nc; ++u) {
-        double t = threadIdx.x < (blockDim.x >> 5) ? red[u][threadIdx.x] : 0.0;
-        for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
-        if (threadIdx.x == 0) part[(long long)(v0 + u) * gridDim.x + blockIdx.x] = t;
-      }
-    }
-    __syncthreads();
+  for (int off = 4; off > 0; off >>= 1) p += __shfl_xor_sync(0xffffffffu, p, off);
+  if ((lane & 7) == 0) red[lane >> 3][warp] = p;
+  __syncthreads();
+  if (warp < nc) {
+    double t = lane < 8 ? red[warp][lane] : 0.0;
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
+    if (lane == 0) part[(long long)(v0 + warp) * gridDim.x + blockIdx.x] = t;
   }
 }
-__global__ void k_dots_final(const double* __restrict__ part, int nv, int nblk, double* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_dots_final(const double* __restrict__ part, int nv, int nblk,
+                                                    double* __restrict__ out) {
   const int v = blockIdx.x;
-  if (v >= nv) return;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   double s = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += part[(long long)v * nblk + b];
-  __shared__ double red[32];
+  for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += __ldcg(part + (long long)v * nblk + b);
+  __shared__ double red[8];
+#pragma unroll
   for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
   if (threadIdx.x < 32) {
-    s = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    s = threadIdx.x < 8 ? red[threadIdx.x] : 0.0;
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
     if (threadIdx.x == 0) out[v] = s;
   }
 }
 stm_status batched_dots(const double* V, int nv, const double* w, long long n, double* out, double* part,
                         int nblk, cudaStream_t s) {
-  k_dots_partial<<<nblk, 256, 0, s>>>(V, nv, w, n, part); note_launch();
-  k_dots_final<<<nv, 256, 0, s>>>(part, nv, nblk, out); note_launch();
+  k_dots_partial<<<dim3(nblk, (nv + 3) / 4), 256, 0, s>>>(V, nv, w, n, part); note_launch();
   STM_CUDA(cudaGetLastError());
+  // launched beside the partial sums, which it waits for
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)nv);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  STM_CUDA(cudaLaunchKernelEx(&cfg, k_dots_final, (const double*)part, nv, nblk, out)); note_launch();
   return STM_OK;
 }
 stm_status vec_norm_sq(const double* x, long long n, double* out, double* part, int nblk, cudaStream_t s) {
