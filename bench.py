@@ -291,17 +291,28 @@ def recorded_traffic(workload_name, kernel, prec=None):
     return None
 
 
-def spmv_roofline(r, wl, sizes, fp64_peak, workload_name):
-    """Dominant kernel of the solve: the node-block FP64 product with the finest J (FP64-pipe bound).
+def spmv_roofline(r, wl, sizes, fp64_peak, workload_name, hbm=None, peak_source=None):
+    """Dominant kernel of the solve: the product with the finest J in FP64 accuracy.
 
-    achieved = 2 * nnz FLOP per launch (one FMA per stored value) / average event time per launch;
-    peak = FP64 FMA throughput measured in the same run (stm_measure_fp64_peak)."""
+    Over FP64 values (small 2D levels) the FP64 pipe is the bound: achieved = 2 * nnz FLOP per launch (one
+    FMA per stored value) / average event time per launch; peak = FP64 FMA throughput measured in the same
+    run (stm_measure_fp64_peak). With hbm given, the level keeps two-limb integers and its bytes are the
+    bound: achieved = algorithmic bytes per launch / the same time, peak = the measured copy bandwidth."""
     f = r["finest"]["jacobian_spmv"]
     if f["ms"] <= 0 or f["launches"] == 0:
         return None
     nnz = sizes[-1]["nnz"]
     us = 1e3 * f["ms"] / f["launches"]
     achieved = 2.0 * nnz / (us * 1e-6) / 1e12
+    if hbm:
+        traffic = recorded_traffic(workload_name, "k_spmv_limbs")
+        gbs = f["bytes"] / (f["ms"] * 1e-3) / 1e9
+        return {"kernel": "k_spmv_limbs (J_g x, finest level, two-limb integers with the exponents of x)",
+                "bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
+                "traffic": traffic["per_launch_bytes"] if traffic else None,
+                "traffic_source": traffic["source"] if traffic else "no capture of the current kernel source",
+                "peak_source": peak_source, "avg_launch_us": us, "fp64_tflops_equivalent": achieved,
+                "fp64_pipe_tflops": fp64_peak, "algorithmic_bytes_per_launch": f["bytes"] / f["launches"]}
     traffic = recorded_traffic(workload_name, "k_spmv_nb_dyn")
     return {"kernel": "k_spmv_nb_dyn (J_g x, finest level, FP64)", "bound": "alu", "achieved": achieved,
             "peak": fp64_peak, "unit": "TFLOP/s", "frac": achieved / fp64_peak if fp64_peak else None,
@@ -311,6 +322,16 @@ def spmv_roofline(r, wl, sizes, fp64_peak, workload_name):
             "flops_per_launch": 2.0 * nnz, "avg_launch_us": us,
             "algorithmic_bytes_per_launch": f["bytes"] / f["launches"],
             "hbm_gbs_algorithmic": f["bytes"] / (f["ms"] * 1e-3) / 1e9}
+
+
+def limb_hbm(wl, hbm=None):
+    """The copy bandwidth where the workload's finest level keeps two-limb integers (3D, 2D dG(2)), else None."""
+    if wl.dim != 3 and wl.k != 2:
+        return None
+    if hbm is None:
+        pk = peaks()
+        hbm = pk["hbm_gbs"] if pk else 6800.0
+    return hbm
 
 
 def defect_roofline(r, sizes, hbm, peak_source, workload_name):
@@ -334,7 +355,8 @@ def defect_roofline(r, sizes, hbm, peak_source, workload_name):
 
 
 def spmm_roofline(f, nnz, fp64_peak, kern, workload_name):
-    """The multi-RHS FP64 SpMM Y = J_g X (32 columns), finest level, FP64-pipe bound.
+    """The multi-RHS SpMM Y = J_g X (32 columns) in FP64 accuracy, finest level, against the FP64 pipe. The
+    product runs on the tensor cores over base-256 digits (3D dG(2) excepted), so the fraction may exceed 1.
 
     achieved = 2 * nnz * 32 FLOP per launch (every stored value meets all 32 columns) / average event
     time per launch; peak = FP64 FMA rate measured in the same run; share = the finest-level SpMM
@@ -345,8 +367,8 @@ def spmm_roofline(f, nnz, fp64_peak, kern, workload_name):
     flops = 2.0 * nnz * 32
     achieved = flops / (us * 1e-6) / 1e12
     total = sum(v["ms"] for v in kern.values())
-    traffic = recorded_traffic(workload_name, "k_spmm_struct")
-    return {"kernel": "k_spmm_struct (Y = J_g X, 32 columns, finest level, FP64)", "bound": "alu",
+    traffic = recorded_traffic(workload_name, "k_spmm_digits")
+    return {"kernel": "k_spmm_digits (Y = J_g X, 32 columns, finest level)", "bound": "alu",
             "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
             "frac": achieved / fp64_peak if fp64_peak else None,
             "traffic": traffic["per_launch_bytes"] if traffic else None,
@@ -665,7 +687,8 @@ def workload_row(args, name, precs, steps, warmup):
            "head": head, "s_per_solve": results[head]["ms_per_solve"] / 1e3,
            "fp64_s": results["f64"]["ms_per_solve"] / 1e3 if "f64" in results else None,
            "by_precision": by_precision_rows(results, errs, steps),
-           "roofline_spmv_f64": {p: spmv_roofline(results[p], wl, sizes, fp64_peak, name) for p in results
+           "roofline_spmv_f64": {p: spmv_roofline(results[p], wl, sizes, fp64_peak, name, limb_hbm(wl), "hbm_gbs")
+                                 for p in results
                                  if split_precision(p)[1] == "f64"}}
     return row
 
@@ -1237,7 +1260,7 @@ def main():
         "gpu_launches": int(r["launches_per_step"] * args.steps),
         "other_rows": rows,
         "roofline": None,
-        "roofline_spmv_f64": spmv_roofline(r, wl, sizes, fp64_peak, args.workload),
+        "roofline_spmv_f64": spmv_roofline(r, wl, sizes, fp64_peak, args.workload, limb_hbm(wl, hbm), peak_src),
         "roofline_defect_f32": defect_roofline(results["bf16+f32d"], sizes, hbm, peak_src, args.workload)
         if "bf16+f32d" in results else None,
         "roofline_vanka_sweep": {"kernel": f"{vk} (y_T = J_T^{{-1}} t_T), finest level, {head} inverses",
