@@ -5,7 +5,7 @@
 // clocks per warp instruction and sub-core the finest 3D dG(1) level (962,208 unknowns, 2.6 GB of values) took
 // 566 us against 382 us for the bytes at the measured copy rate. Here J's velocity rows are two-limb integers
 // (limbs.h, eight bytes per value as before), three integer multiply-adds each, 13 clocks: the bytes are the limit
-// again, and 427 us are 6.2 TB/s of what is read. On smaller 3D levels: 91.7 -> 71.1 us (127,920 unknowns),
+// again: 425 us are 6.1 TB/s of values, 6.6 TB/s of what is read (padded runs read 5 % more sectors). On smaller 3D levels: 91.7 -> 71.1 us (127,920 unknowns),
 // 49.9 -> 32.4 (18,000); 3D dG(0) 175.8 -> 145 (481,104), dG(2) 651 -> 469 (735,369); 2D dG(2) 89.3 -> 78.8
 // (536,448) and 35.1 -> 31.0 (135,168).
 //   - Row exponents come with the values; the exponent of x is that of the largest entry around a node, found per
