@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_cell_inverse(const
         widx[warp] = bi;
       }
       __syncthreads();
+      bool singular = false;  // the same for all threads: read between two barriers that enclose no write
       for (int k = 0; k < w; ++k) {
         const int gk = p0 + k;
         if (warp == 0) {
@@ -198,7 +199,8 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_cell_inverse(const
           }
         }
         __syncthreads();
-        if (s_bad) break;
+        singular = s_bad != 0;
+        if (singular) break;
         const int p = s_piv;
         const double u = ubuf[j16];
         bk = -1;
@@ -238,7 +240,8 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_cell_inverse(const
         }
         __syncthreads();
       }
-      if (s_bad) break;
+      // not s_bad: threads that are through the pivots may already set it for a row of M that is not finite
+      if (singular) break;
       // M back into the matrix and as a row operand: a warp per 16-row tile, lane = (row, position pairs)
       for (int e = tid; e < n * w; e += kThreads) {
         const int j = e / n, i = e - j * n;
