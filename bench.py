@@ -325,8 +325,8 @@ def spmv_roofline(r, wl, sizes, fp64_peak, workload_name, hbm=None, peak_source=
 
 
 def limb_hbm(wl, hbm=None):
-    """The copy bandwidth where the workload's finest level keeps two-limb integers (3D, 2D dG(2)), else None."""
-    if wl.dim != 3 and wl.k != 2:
+    """The copy bandwidth where the workload's finest level keeps two-limb integers (3D), else None."""
+    if wl.dim != 3:
         return None
     if hbm is None:
         pk = peaks()

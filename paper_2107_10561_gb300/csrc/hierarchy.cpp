@@ -504,8 +504,8 @@ static stm_status build_level(const stm_params& p, int g, Level& L, std::vector<
       lbase[nd + 1] = lbase[nd] + (long long)(L.K * d) * (L.K * d * up(nn[nd]) + up((long long)np * ncell[nd]));
     L.nval_cap = lbase[R];
     STM_TRY(upload(&L.lbase, lbase));
-    STM_CUDA(cudaMalloc((void**)&L.nexp, sizeof(int) * (size_t)R * (L.K * d + 1)));
-    STM_CUDA(cudaMalloc((void**)&L.cexp, sizeof(int2) * C));
+    STM_CUDA(cudaMalloc((void**)&L.nexp, limb_node_exps(L)));
+    STM_CUDA(cudaMalloc((void**)&L.cexp, limb_cell_exps(L)));
   }
   STM_CUDA(cudaMalloc((void**)&L.nval, sizeof(double) * L.nval_cap));
   {

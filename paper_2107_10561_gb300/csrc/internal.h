@@ -183,11 +183,11 @@ struct Level {
   double* pvalT = nullptr;
   double *nvalJT = nullptr, *pvalJT = nullptr;  // the same two copies for J^T (built with valT)
   // limb_lanes > 0: nval and nvalJT hold two-limb integers instead (limbs.h), positions in runs of limb_lanes;
-  // per node the K*d row exponents and the offset of the pressure columns; cexp: per cell, x's exponents
+  // per node the exponents of J by component of the row and class of the column, and by row; per cell those of x by class
   int limb_lanes = 0;
   long long* lbase = nullptr;              // [R+1] start of each node, in values
-  int *nexp = nullptr, *nexpJT = nullptr;  // [R][K*d + 1]
-  int2* cexp = nullptr;                    // [C]
+  short *nexp = nullptr, *nexpJT = nullptr;  // [R]
+  short* cexp = nullptr;                     // [C][padded]
   unsigned* spmv_work = nullptr;  // [2] unit counter and finished-CTA count of the FP64 product (zeroed)
   // FP32 copies of nval/pvalT (and of nvalJT/pvalJT) in the same layout, for the V-cycle's defects
   // r - J_g d with defect_precision = STM_F32; null otherwise
@@ -406,7 +406,9 @@ int limb_lanes(const Level& L);
 // the same product of the levels that keep limbs, and their copy of the velocity rows (kernels_limb_spmv.cu)
 stm_status spmv_limbs(const Level& L, int transpose, const double* x, const double* b, double* y, int mode,
                       cudaStream_t s, const int* jobs, int njobs);
-stm_status build_limbs(const Level& L, const double* val, double* nval, int* nexp, cudaStream_t s);
+stm_status build_limbs(const Level& L, const double* val, double* nval, short* nexp, cudaStream_t s);
+size_t limb_node_exps(const Level& L);  // bytes of nexp and of cexp
+size_t limb_cell_exps(const Level& L);
 // node-block and warp-transposed pressure-row copies of J's or J^T's values
 stm_status build_nodeblock(const Level& L, int transpose, cudaStream_t s);
 // y = b - J_g x (transpose: J_g^T) over the FP32 copies of the values: x rounded to FP32 into L.x32

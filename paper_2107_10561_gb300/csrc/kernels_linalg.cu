@@ -112,7 +112,7 @@ stm_status ensure_transpose(Hierarchy& H, int g, cudaStream_t s) {
   STM_CUDA(cudaMalloc(&L.nvalJT, sizeof(double) * L.nval_cap));
   STM_CUDA(cudaMalloc(&L.pvalJT, sizeof(double) * L.pval_len));
   STM_CUDA(cudaMemsetAsync(L.pvalJT, 0, sizeof(double) * L.pval_len, s));
-  if (L.limb_lanes) STM_CUDA(cudaMalloc(&L.nexpJT, sizeof(int) * L.R * (L.K * L.dim + 1)));
+  if (L.limb_lanes) STM_CUDA(cudaMalloc(&L.nexpJT, limb_node_exps(L)));
   STM_TRY(build_nodeblock(L, 1, s));
   if (H.p.defect_precision == STM_F32) STM_TRY(build_values_f32(L, 1, s));
   return STM_OK;

@@ -16,8 +16,7 @@
 //   - warp-transposed pressure rows: one lane per row, entry t of 32 consecutive rows contiguous.
 // Column indices are never read. In FP64, issue slots of the FP64 pipe are the limit (one FP64 warp
 // instruction every 16 cycles per SM); results equal the plain CSR product up to FP64 summation
-// order. FP64 values are kept on 2D levels only, and there where limb_lanes() says so: the others' velocity
-// rows are integers (kernels_limb_spmv.cu). In FP32 the arithmetic is cheap and the loads in flight per SM set the pace.
+// order. FP64 values are kept on 2D levels only: the velocity rows of 3D levels are integers (kernels_limb_spmv.cu). In FP32 the arithmetic is cheap and the loads in flight per SM set the pace.
 #include "internal.h"
 
 namespace stm {
@@ -584,6 +583,7 @@ stm_status spmv_nodeblock(const Level& L, int transpose, const double* x, const 
   switch (L.dim * 10 + L.K + cls) {
     case 21: return launch_nb_dyn<4, 1, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
     case 22: return launch_nb_dyn<4, 2, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
+    case 23: return launch_nb_dyn<4, 3, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
     case 121: return launch_nb_dyn<16, 1, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
     case 122: return launch_nb_dyn<16, 2, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
     case 123: return launch_nb_dyn<16, 3, 2, 1>(L, nval, pvalT, x, b, y, mode, s, jobs, njobs);
