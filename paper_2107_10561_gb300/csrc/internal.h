@@ -209,7 +209,7 @@ struct Level {
   // smoother data (levels >= 1)
   void* inv = nullptr;            // [C][n*n] column-major per cell, storage precision
   int2* lim = nullptr;            // FP64 inverses once more as two-limb integers, same layout (null: no room)
-  int* lexp = nullptr;            // [C][n+1] the exponents of their rows, the offset of the pressure columns
+  short* lexp = nullptr;          // [C][classes of columns][ld] the exponents of their rows by class
   double* wmult = nullptr;        // [N] 1/m_i
   int* own_ptr = nullptr;         // [N+1]
   int* own_pos = nullptr;         // [sum m_i] flat positions c*n + alpha
@@ -355,10 +355,11 @@ stm_status launch_fill_colidx(Level& Lv, const int* nbr_ptr, const int* nbr_idx,
 stm_status inject_linearisation(Hierarchy& H, const double* X_fine, cudaStream_t s);
 stm_status assemble_level(Hierarchy& H, int g, double nu, cudaStream_t s);
 stm_status factor_level(Hierarchy& H, int g, cudaStream_t s);
-// FP64 inverses: their copy in limbs and the cell solves with it (kernels_limb_vanka.cu)
-stm_status inverse_limbs(Level& L, cudaStream_t s);
-stm_status vanka_limbs(const Level& L, const double* t, const int* cells, int nc, int transpose, double* scatter,
-                       double omega, cudaStream_t s);
+// FP64 inverses: their copy in limbs and the cell solves with it (kernels_limb_vanka.cu), for nc cells at a time
+bool limb_cells_pay(int nc);
+stm_status inverse_limbs(Level& L, int nc, cudaStream_t s);
+stm_status vanka_limbs(const Level& L, const double* t, const int* cells, int nc, double* scatter, double omega,
+                       cudaStream_t s);
 stm_status factor_coarse(Hierarchy& H, cudaStream_t s);
 stm_status ensure_transpose(Hierarchy& H, int g, cudaStream_t s);
 // Dense FP64 products and inverses on the tensor cores (kernels_dense.cu). An operand is cut into digits in

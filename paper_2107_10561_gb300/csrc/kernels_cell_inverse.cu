@@ -435,7 +435,9 @@ stm_status factor_level(Hierarchy& H, int g, cudaStream_t s) {
   a.scratch = in_smem ? nullptr : H.cell_scratch;
   if (per_sm == 4) STM_TRY(launch<128>(H, a, L.inv, blocks, smem, s));
   else STM_TRY(launch<256>(H, a, L.inv, blocks, smem, s));
-  return H.p.inv_precision == STM_F64 ? inverse_limbs(L, s) : STM_OK;
+  // the coloured smoother solves on the cells of one colour at a time
+  const int nc = H.p.smoother == STM_VANKA_COLOURED ? L.C >> L.dim : L.C;
+  return H.p.inv_precision == STM_F64 ? inverse_limbs(L, nc, s) : STM_OK;
 }
 
 }  // namespace stm

@@ -1,21 +1,27 @@
-// Cell solves y_T = J_T^{-1} t_T (or with the transpose) over FP64 inverses, on the INT32 pipe.
+// Cell solves y_T = J_T^{-1} t_T over FP64 inverses, on the INT32 pipe, every row as accurate as an FP64 sum of it is held
+// to be.
 //
-// Every entry of an inverse is read once and needs one multiply-add; in FP64 that takes 74 clocks per warp
-// instruction and sub-core, while HBM delivers the next 256 bytes after 44. The inverses are therefore kept a second
-// time as two-limb integers (limbs.h), each row at a scale of its own, which takes 13 clocks. On 16,128 cells of 2D
-// dG(2) (528 MB) a launch takes 91 us, 76 % of the copy rate, where the FP64 kernel took 150; whole sweeps: 243 ->
-// 181 us, 2D dG(1) 156 -> 104, 3D dG(0) 449 -> 375, 3D dG(1) (2,016 cells) 195 -> 159. Cutting the FP64 values into
-// limbs as they are read instead took 126 us.
+// Every entry of an inverse is read once and needs one multiply-add; in FP64 that is the limit (2D dG(2), 16,384 cells,
+// 528 MB: 150 us against 78 us for the bytes at the measured copy rate). The inverses are therefore kept a second time as
+// two-limb integers (limbs.h), three integer multiply-adds each: 105 us; 2D dG(1) 97 -> 65 us, 3D dG(0) 280 -> 219,
+// 3D dG(1) (2,048 cells) 115 -> 108.
+//   - A sum of integers has one scale. An inverse has an exponent per row and class of columns (a velocity component or
+//     the pressures of one time node), t one per class; a class's columns are summed at the product of the two and the
+//     sum is shifted to the largest such product of the row. What is cut off is 2^-57 of that product. The classes'
+//     sums bound |J_T^{-1}||t| from below: a row where they stay 2^-kSpare below the largest product is summed again
+//     in FP64. kSpare = 8 keeps what one term may lose (2^-56.4) below m 2^-53 |J_T^{-1}||t|, the bound of an FP64 chain of
+//     m >= 42 terms. Right-hand sides and residuals have no such row in 2D, one in 100 cells in 3D dG(1) and one in 20
+//     to 50 in 3D dG(0). With one scale per row and one offset for the pressures (91 us) the error was 3 to 400 times
+//     that of FP64 (normally distributed t, tau 1e-2 to 1e-5).
 //   - A warp per cell, whole lines per load; lanes own row pairs and t's limbs are broadcast from shared memory, so
-//     a column costs a load, a shared load and six multiply-adds per lane. Several warps per cell (each a block of
-//     columns, sums joined in FP64) where cells are fewer than resident warps.
-//   - t is cut below the largest entry of the cell, the pressure columns with one offset per cell against the
-//     velocity columns. Against the FP64 kernel results differ by 2e-16 to 1e-15 of the largest entry.
-//   - The transpose goes a thread per column (2D dG(2) 236 us as in FP64, 3D dG(0) 413 -> 384, dG(1) 217 -> 186).
-//   - Cells with an infinity, a NaN or a scale near the ends of the exponent range, in the inverse or in t, are
-//     summed in FP64 from the FP64 inverses, which the 32-column products and the copy to the host read anyway.
-//   - Cells of fewer than 32 rows (2D dG(0): 21) stay with the FP64 kernel: 11 of 32 lanes would own rows (63 against
-//     65 us per sweep, and 38 against 35 on 4,032 cells). So do levels without room for the second copy.
+//     a column costs a load, a shared load and six multiply-adds per lane. Exponents and the first columns are on their
+//     way while t is cut.
+//   - Fewer cells than four fifths of the resident warps (1,945) stay with the FP64 kernel, which takes several warps per
+//     cell (3D dG(1), 1,536 cells, whole sweep: 185 against 168 us; with several warps here 360 cells took 46 us against
+//     31), and so does the transpose (2D dG(2): 204 us against 145; the scales of its products differ from row to row of
+//     the inverse and class of columns). So do cells of fewer than 32 rows (2D dG(0): 21) and levels without
+//     room for the second copy.
+//   - Cells with an infinity or a NaN, in the inverse or in t, are summed in FP64 from the FP64 inverses.
 #include "digits.h"
 #include "internal.h"
 #include "limbs.h"
@@ -23,86 +29,106 @@
 namespace stm {
 namespace {
 
-constexpr int kNone = -(1 << 20);  // biased exponent where every entry is zero
-constexpr int kPlain = 1 << 20;    // pressure offset of a cell whose inverse holds an infinity, a NaN or tiny rows
+constexpr int kNone = -20000;  // exponent where every entry is zero (16 bits)
+constexpr int kPlain = 20000;  // exponent of a row's class that holds an infinity or a NaN
+constexpr int kCtas = 2;       // per SM, of eight warps
+constexpr int kSpare = 8;      // bits by which a row's sum of magnitudes may lie below its scale
 
-__device__ __forceinline__ int biased(double v) {
-  const int hi = __double2hiint(v) & 0x7FFFFFFF;
-  return (hi | __double2loint(v)) == 0 ? kNone : hi >> 20;
+// The columns of a cell by class: per time node the D velocity components, then the pressures.
+template <int K, int D>
+struct Cell {
+  static constexpr int NV = D == 2 ? 9 : 27, NP = D + 1, NT = D * NV + NP, PT = D + 1;  // PT classes per time node
+  static constexpr int n = K * NT, nk = K * PT;
+  // batches of three columns, within a class each: the last one of a time node is short in 3D
+  static constexpr int BT = (D * NV + NP + 2) / 3, batches = K * BT;
+  static __device__ __forceinline__ int column(int b) { return b / BT * NT + b % BT * 3; }
+  static __device__ __forceinline__ int width(int b) { return min(3, NT - b % BT * 3); }
+  static __device__ __forceinline__ bool last(int b) { return b % BT == BT - 1 || (b % BT < D * NV / 3 && b % BT % (NV / 3) == NV / 3 - 1); }
+  static __device__ __forceinline__ int cls(int j) {
+    const int a = j / NT, r = j - a * NT;
+    return a * PT + min(r / NV, D);
+  }
+  static __device__ __forceinline__ int begin(int k) { return k / PT * NT + k % PT * NV; }
+};
+
+__device__ __forceinline__ int exponent_of(double v) {
+  const int e = exp_above(v);
+  return e == kExpZero ? kNone : e > 1024 ? kPlain : e;
 }
 
-// Limbs of a cell's inverse in the layout of the inverse, each row at the biased exponent of its largest velocity
-// column, the pressure columns delta above; lexp: [C][n + 1], the rows' exponents and delta. One CTA per cell.
-__global__ void __launch_bounds__(256) k_inverse_limbs(const double* __restrict__ inv, int n, int ld, int nt, int nvel,
-                                                       int2* __restrict__ out, int* __restrict__ lexp) {
-  __shared__ int row[256], offset, bad;
+// Limbs of a cell's inverse in the layout of the inverse; lexp: [C][classes][ld], the exponents. One CTA per cell.
+template <int K, int D>
+__global__ void __launch_bounds__(256) k_inverse_limbs(const double* __restrict__ inv, int ld, int2* __restrict__ out,
+                                                       short* __restrict__ lexp) {
+  using S = Cell<K, D>;
+  constexpr int n = S::n, nk = S::nk;
+  __shared__ short ex[nk][256];
   const int c = blockIdx.x, i = threadIdx.x;
   const double* M = inv + (size_t)c * n * ld;
-  if (i == 0) offset = kNone, bad = 0;
-  __syncthreads();
-  if (i < n) {
-    int ev = kNone, ep = kNone;
-    for (int k = 0, r = 0; k < n; ++k) {
-      const int e = biased(M[(size_t)k * ld + i]);
-      if (r < nvel) ev = max(ev, e);
-      else ep = max(ep, e);
-      if (++r == nt) r = 0;
+  if (i < ld) {
+    for (int k = 0; k < nk; ++k) {
+      int e = kNone;
+      const int end = k + 1 < nk ? S::begin(k + 1) : n;
+      if (i < n)
+        for (int j = S::begin(k); j < end; ++j) e = max(e, exponent_of(M[(size_t)j * ld + i]));
+      ex[k][i] = (short)e;
+      lexp[((size_t)c * nk + k) * ld + i] = (short)e;
     }
-    const int most = max(ev, ep);
-    if (most >= 2047 || (most != kNone && most < 128)) bad = 1;
-    if (ev == kNone) ev = ep == kNone ? 1023 : ep;
-    if (ep != kNone) atomicMax(&offset, ep - ev);
-    row[i] = ev;
   }
   __syncthreads();
-  const int delta = offset == kNone ? 0 : offset;
-  const bool plain = bad || delta > 900 || delta < -900;
-  if (i < n) lexp[(size_t)c * (n + 1) + i] = row[i];
-  if (i == 0) lexp[(size_t)c * (n + 1) + n] = plain ? kPlain : delta;
   for (int e = i; e < n * ld; e += 256) {
-    const int j = e / ld, r = e - j * ld;
-    const bool zero = plain || r >= n;
-    out[(size_t)c * n * ld + e] =
-        limbs_of(zero ? 0.0 : M[e], zero ? 0 : row[r] - 1022 + (j % nt < nvel ? 0 : delta));
+    const int j = e / ld, r = e - j * ld, x = ex[S::cls(j)][r];
+    out[(size_t)c * n * ld + e] = x == kNone || x == kPlain ? make_int2(0, 0) : limbs_of(M[e], x);
   }
 }
 
-// The largest exponents of t's velocities and pressures give the exponent that t is cut at, or kPlain.
-__device__ __forceinline__ int common_top(int ev, int ep, int delta) {
-  if (delta == kPlain) return kPlain;
-  const int most = max(ev, ep);
-  if (most == kNone) return 1023;
-  const int top = max(ev, ep + delta);
-  return most >= 2047 || min(top, top - delta) < 64 || max(top, top - delta) > 2046 ? kPlain : top;
-}
-__device__ __forceinline__ void carry(long long& h, long long& m) {
-  h += m >> kLimbBits;
-  m &= (1ll << kLimbBits) - 1;
-}
 __device__ __forceinline__ double join(long long h, long long m) { return fma((double)h, (double)(1ll << kLimbBits), (double)m); }
-__device__ __forceinline__ int scale_exp(int row, int top) { return row + top - 2044 - (2 * kLimbTotal - kLimbBits); }
+// The exponent of a sum of limb products at the scale 2^top
+__device__ __forceinline__ int scale_exp(int top) { return top - (2 * kLimbTotal - kLimbBits); }
 
-// G warps per cell (8 / G cells per CTA), each a block of columns. Lane l of a warp owns the row pairs
-// l, l + 32, .. (NR of them); UB columns are in flight, t's limbs stand in the warp's own shared memory. The next cell's t is gathered while the present one is streamed.
-template <int NR>
-__global__ void __launch_bounds__(256, NR <= 2 ? 3 : 2) k_limb_cells(const int4* __restrict__ lim, const int* __restrict__ lexp,
+// (H, M) += (h, m) >> sh, 0 <= sh; returns the part of it in units of H
+__device__ __forceinline__ long long merge(long long h, long long m, int sh, long long& H, long long& M) {
+  constexpr unsigned mask = (1u << kLimbBits) - 1;
+  h += m >> kLimbBits;
+  unsigned lo = (unsigned)m & mask;
+  for (; sh >= kLimbBits; sh -= kLimbBits) {  // classes that hardly matter
+    lo = (unsigned)h & mask;
+    h >>= kLimbBits;
+  }
+  M += (((unsigned)h << (kLimbBits - sh)) & mask) | (lo >> sh);
+  h >>= sh;
+  H += h;
+  return h;
+}
+
+// One row in plain FP64
+__device__ __forceinline__ double plain_row(const double* M, const int* ic, const double* t, int n, int stride) {
+  double y = 0.0;
+#pragma unroll 8
+  for (int j = 0; j < n; ++j) y = fma(M[(size_t)j * stride], t[ic[j]], y);
+  return y;
+}
+
+// A warp per cell, eight cells per CTA. Lane l of a warp owns the row pairs l, l + 32, .. (NR of them); batches of three
+// columns are loaded PD - 1 ahead, t's limbs stand in the warp's own shared memory. The next cell's t is gathered while
+// the present one is streamed.
+template <int K, int D>
+__global__ void __launch_bounds__(256, kCtas) k_limb_cells(const int4* __restrict__ lim, const short* __restrict__ lexp,
                                                        const double* __restrict__ inv, const int* __restrict__ idx,
                                                        const double* __restrict__ t, double* __restrict__ Y,
-                                                       const int* __restrict__ cell_list, int ncells, int n, int ld, int G,
-                                                       int nt, int nvel, double* __restrict__ d_scatter, double omega) {
-  constexpr int UB = NR == 1 ? 6 : NR < 4 ? 3 : 2, NT = 2 * NR;
-  // h grows by less than 2^56 per column: t is cut a bit higher where a warp may see more than 127
-  constexpr int kLess = NR > 1 ? 1 : 0;
-  constexpr int kEvery = (21 - UB) / UB;  // batches between carries: m grows by up to 1.5 x 2^58 per column
+                                                       const int* __restrict__ cell_list, int ncells, int ld,
+                                                       double* __restrict__ d_scatter, double omega) {
+  using S = Cell<K, D>;
+  constexpr int n = S::n, nk = S::nk, NR = (n + 63) / 64, NT = 2 * NR, PD = NR == 1 ? 4 : NR == 2 ? 2 : 1;
+  // a class's sums stay below 2^63: 27 columns of 2^56 in h and 2^58 in m
+  static_assert(S::NV <= 31, "m overflows");
   __shared__ double2 tsh[8][32 * NR];
-  __shared__ double part[8][64 * NR];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = warp & (G - 1), LDV = ld / 2;
-  const int slots = 8 / G, slot = warp / G;
+  __shared__ int te[8][nk];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, LDV = ld / 2;
   int2* tl = reinterpret_cast<int2*>(tsh[warp]);
-  double* td = reinterpret_cast<double*>(tsh[warp]);
-  unsigned vel = 0;
+  int cls[NT];
 #pragma unroll
-  for (int k = 0; k < NT; ++k) vel |= (unsigned)((lane + 32 * k) % nt < nvel) << k;
+  for (int k = 0; k < NT; ++k) cls[k] = S::cls(min(lane + 32 * k, n - 1));
   auto cell_of = [&](int ci) { return ci < ncells ? (cell_list ? cell_list[ci] : ci) : -1; };
   double tv[NT];
   int at[NT];
@@ -114,268 +140,174 @@ __global__ void __launch_bounds__(256, NR <= 2 ? 3 : 2) k_limb_cells(const int4*
 #pragma unroll
     for (int k = 0; k < NT; ++k) tv[k] = at[k] >= 0 ? t[at[k]] : 0.0;
   };
-  // the warp's columns; lanes beyond the rows repeat the last pair
-  const int cb = (n + G - 1) / G, j0 = min(g * cb, n), cols = min(cb, n - j0);
-  unsigned off[NR];
+  unsigned off[NR];  // lanes beyond the rows repeat the last pair
 #pragma unroll
-  for (int r = 0; r < NR; ++r) off[r] = (unsigned)(j0 * LDV + min(lane + 32 * r, LDV - 1));
-  const int step = gridDim.x * slots;
-  int ci = blockIdx.x * slots + slot, c = cell_of(ci);
+  for (int r = 0; r < NR; ++r) off[r] = (unsigned)min(lane + 32 * r, LDV - 1);
+  const int step = gridDim.x * 8;
+  int ci = blockIdx.x * 8 + warp, c = cell_of(ci);
   lookup(c);
   gather();
-  for (; ci - slot < ncells; ci += step) {  // the same for all warps of a CTA
-    const bool has = c >= 0;
-    const int* ie = lexp + (size_t)(has ? c : 0) * (n + 1);
-    const int delta = ie[n];
-    int ev = kNone, ep = kNone;
+  for (; c >= 0; ci += step) {
+    const int4* A = lim + (size_t)c * n * LDV;
+    int4 raw[PD][3][NR];
+    auto load = [&](int b, int4 (*to)[NR]) {
+      const int w = b < S::batches ? S::width(b) : 0;
+      const int4* col = A + (unsigned)(S::column(b) * LDV);
 #pragma unroll
-    for (int k = 0; k < NT; ++k) {
-      const int e = biased(tv[k]);
-      if (vel >> k & 1) ev = max(ev, e);
-      else ep = max(ep, e);
+      for (int u = 0; u < 3; ++u)
+        if (u < w)
+#pragma unroll
+          for (int r = 0; r < NR; ++r) to[u][r] = __ldcs(col + u * LDV + off[r]);
+    };
+#pragma unroll
+    for (int p = 0; p < PD - 1; ++p) load(p, raw[p]);
+    // t's exponents by class, the scale of the lane's rows
+    const short2* ex = reinterpret_cast<const short2*>(lexp + (size_t)c * nk * ld);
+    short2 x[nk][NR];
+#pragma unroll
+    for (int k = 0; k < nk; ++k)
+#pragma unroll
+      for (int r = 0; r < NR; ++r) x[k][r] = __ldg(ex + k * LDV + off[r]);
+    int e[NT];
+#pragma unroll
+    for (int k = 0; k < NT; ++k) e[k] = exponent_of(tv[k]);
+    int top[NR][2];
+    bool plain = false;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) top[r][0] = top[r][1] = 2 * kNone;
+#pragma unroll
+    for (int k = 0; k < nk; ++k) {
+      int v = kNone;
+#pragma unroll
+      for (int q = 0; q < NT; ++q)
+        if (cls[q] == k) v = max(v, e[q]);
+      v = __reduce_max_sync(0xffffffffu, v);
+      if (lane == 0) te[warp][k] = v;
+      plain = plain || v == kPlain;
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        plain = plain || x[k][r].x == kPlain || x[k][r].y == kPlain;
+        top[r][0] = max(top[r][0], x[k][r].x + v);
+        top[r][1] = max(top[r][1], x[k][r].y + v);
+      }
     }
-    ev = __reduce_max_sync(0xffffffffu, ev);
-    ep = __reduce_max_sync(0xffffffffu, ep);
-    const int top = common_top(ev, ep, delta);
+    plain = __any_sync(0xffffffffu, plain);
     __syncwarp();
 #pragma unroll
-    for (int k = 0; k < NT; ++k) {
-      if (top != kPlain) tl[lane + 32 * k] = limbs_below(tv[k], (vel >> k & 1 ? top : top - delta) + kLess);
-      else td[lane + 32 * k] = tv[k];
-    }
+    for (int k = 0; k < NT; ++k) tl[lane + 32 * k] = plain || e[k] == kNone ? make_int2(0, 0) : limbs_of(tv[k], te[warp][cls[k]]);
     __syncwarp();
     const int cn = cell_of(ci + step);
     lookup(cn);
-    double a[NR][2];
+    long long H[NR][2], M[NR][2], h[NR][2], m[NR][2];
+    unsigned sum[NR][2];
 #pragma unroll
-    for (int r = 0; r < NR; ++r) a[r][0] = a[r][1] = 0.0;
-    if (has && top != kPlain) {
-      long long h[NR][2], m[NR][2];
+    for (int r = 0; r < NR; ++r)
 #pragma unroll
-      for (int r = 0; r < NR; ++r) h[r][0] = h[r][1] = m[r][0] = m[r][1] = 0;
-      const int4* M = lim + (size_t)c * n * LDV;
-      const int2* tx = tl + j0;
-      auto columns = [&](int cnt) {  // cnt <= UB: constant after unrolling but for the last batch
-        int4 raw[UB][NR];
+      for (int v = 0; v < 2; ++v) H[r][v] = M[r][v] = h[r][v] = m[r][v] = 0, sum[r][v] = 0;
+    if (!plain) {
+#pragma unroll 1
+      for (int bb = 0; bb < S::batches; bb += PD)
 #pragma unroll
-        for (int u = 0; u < UB; ++u)
-          if (u < cnt)
+        for (int p = 0; p < PD; ++p) {
+          const int b = bb + p;
+          if (b >= S::batches) break;
+          load(b + PD - 1, raw[(p + PD - 1) % PD]);
+          const int w = S::width(b), j = S::column(b);
 #pragma unroll
-            for (int r = 0; r < NR; ++r) raw[u][r] = __ldcs(M + (off[r] + (unsigned)(u * LDV)));
+          for (int u = 0; u < 3; ++u)
+            if (u < w) {
+              const int2 y = tl[j + u];
 #pragma unroll
-        for (int u = 0; u < UB; ++u)
-          if (u < cnt) {
-            const int2 x = tx[u];
+              for (int r = 0; r < NR; ++r) {
+                limb_fma(make_int2(raw[p][u][r].x, raw[p][u][r].y), y, h[r][0], m[r][0]);
+                limb_fma(make_int2(raw[p][u][r].z, raw[p][u][r].w), y, h[r][1], m[r][1]);
+              }
+            }
+          if (S::last(b)) {
+            const int k = S::cls(j), tk = te[warp][k];
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
-              limb_fma(make_int2(raw[u][r].x, raw[u][r].y), x, h[r][0], m[r][0]);
-              limb_fma(make_int2(raw[u][r].z, raw[u][r].w), x, h[r][1], m[r][1]);
+              const short2 z = __ldg(ex + k * LDV + off[r]);
+#pragma unroll
+              for (int v = 0; v < 2; ++v) {
+                // one bit lower than the scale, so that 254 columns fit
+                const long long q = merge(h[r][v], m[r][v], min(top[r][v] + 1 - (v ? z.y : z.x) - tk, 4 * kLimbBits), H[r][v], M[r][v]);
+                sum[r][v] += (unsigned)abs((int)(q >> 32));
+                h[r][v] = m[r][v] = 0;
+              }
             }
           }
-      };
-      int k = 0, left = cols;
-#pragma unroll 1
-      for (; left >= UB; left -= UB) {
-        columns(UB);
-        M += UB * LDV;
-        tx += UB;
-        if (++k < kEvery) continue;
-        k = 0;
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-          carry(h[r][0], m[r][0]);
-          carry(h[r][1], m[r][1]);
         }
-      }
-#pragma unroll 1
-      for (; left > 0; --left) {
-        columns(1);
-        M += LDV;
-        ++tx;
-      }
-#pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        a[r][0] = join(h[r][0], m[r][0]);
-        a[r][1] = join(h[r][1], m[r][1]);
-      }
-    } else {
-      if (has) {
-        const double* M = inv + (size_t)c * n * ld;
-        for (int j = j0; j < j0 + cols; ++j)
-#pragma unroll
-          for (int r = 0; r < NR; ++r)
-            if (lane + 32 * r < LDV) {
-              a[r][0] = fma(M[(size_t)j * ld + 2 * (lane + 32 * r)], td[j], a[r][0]);
-              a[r][1] = fma(M[(size_t)j * ld + 2 * (lane + 32 * r) + 1], td[j], a[r][1]);
-            }
-      }
     }
     gather();
-    if (G > 1) {
-      __syncthreads();
 #pragma unroll
-      for (int r = 0; r < NR; ++r) *reinterpret_cast<double2*>(part[warp] + 2 * (lane + 32 * r)) = make_double2(a[r][0], a[r][1]);
-      __syncthreads();
-      // warp g of the cell finishes the row pairs g (mod G)
-    }
-    if (has)
+    for (int r = 0; r < NR; ++r)
 #pragma unroll
-      for (int r = 0; r < NR; ++r)
-#pragma unroll
-        for (int v = 0; v < 2; ++v) {
-          const int i = 2 * (lane + 32 * r) + v;
-          if (i >= n || (lane & (G - 1)) != g) continue;
-          double y = a[r][v];
-          if (G > 1) {
-            y = 0.0;
-            for (int w = 0; w < G; ++w) y += part[slot * G + w][i];
-          }
-          if (top != kPlain) y = scale_pow2(y, scale_exp(ie[i], top + kLess));
-          if (d_scatter) d_scatter[idx[(long long)c * n + i]] += omega * y;
-          else Y[(long long)c * n + i] = y;
-        }
+      for (int v = 0; v < 2; ++v) {
+        const int i = 2 * (lane + 32 * r) + v;
+        if (i >= n) continue;
+        double y = scale_pow2(join(H[r][v], M[r][v]), scale_exp(top[r][v] + 1));
+        if (top[r][v] < kNone / 2) y = 0.0;  // the row or all entries that it meets are zero
+        else if (plain || sum[r][v] < (1u << (23 - kSpare)))
+          y = plain_row(inv + (size_t)c * n * ld + i, idx + (long long)c * n, t, n, ld);
+        if (d_scatter) d_scatter[idx[(long long)c * n + i]] += omega * y;
+        else Y[(long long)c * n + i] = y;
+      }
     c = cn;
   }
 }
 
-// The transpose: a thread per column, which it streams along its rows; P cells per CTA of T threads. The rows'
-// exponents go into t's.
-__global__ void __launch_bounds__(256, 4) k_limb_cells_t(const int4* __restrict__ lim, const int* __restrict__ lexp,
-                                                         const double* __restrict__ inv, const int* __restrict__ idx,
-                                                         const double* __restrict__ t, double* __restrict__ Y,
-                                                         const int* __restrict__ cell_list, int ncells, int n, int ld,
-                                                         int T, int P, int nt, int nvel, double* __restrict__ d_scatter,
-                                                         double omega) {
-  constexpr int UB = 6;
-  extern __shared__ int4 sm4[];  // [P][ld] limbs of t
-  __shared__ int most[16], worst[16];
-  const int slot = threadIdx.x / T, j = threadIdx.x - slot * T, LDV = ld / 2;
-  int2* tl = reinterpret_cast<int2*>(sm4) + slot * ld;
-  double* td = reinterpret_cast<double*>(tl);
-  for (int base = blockIdx.x * P; base < ncells; base += gridDim.x * P) {
-    const int ci = base + slot;
-    const bool has = slot < P && ci < ncells;
-    const int c = has ? (cell_list ? cell_list[ci] : ci) : 0;
-    const int* ic = idx + (long long)c * n;
-    const int* ie = lexp + (size_t)c * (n + 1);
-    __syncthreads();
-    if (threadIdx.x < 16) most[threadIdx.x] = worst[threadIdx.x] = kNone;
-    __syncthreads();
-    if (has)
-      for (int i = j; i < ld; i += T) {
-        const double v = i < n ? t[ic[i]] : 0.0;
-        td[i] = v;
-        const int e = biased(v);
-        if (e != kNone) {
-          atomicMax(&most[slot], e + ie[i]);
-          atomicMax(&worst[slot], e < 64 ? 2047 : e);
-        }
-      }
-    __syncthreads();
-    const int delta = ie[n], all = has ? most[slot] : kNone;  // largest product of a row's scale and t's entry
-    const bool plain = delta == kPlain || (all != kNone && (worst[slot] >= 2047 || all < 256));
-    if (has && !plain)
-      for (int i = j; i < ld; i += T) {
-        const int top = all == kNone || i >= n ? 1023 : all - ie[i];  // below 64 only where t is zero
-        tl[i] = top < 64 ? make_int2(0, 0) : limbs_below(td[i], top);
-      }
-    __syncthreads();
-    if (has && j < n) {
-      double y = 0.0;
-      if (!plain) {
-        const int4* col = lim + ((size_t)c * n + j) * LDV;
-        long long h = 0, m = 0, hs = 0;
-        for (int i0 = 0; i0 < LDV; i0 += UB) {
-          int4 raw[UB];
-#pragma unroll
-          for (int u = 0; u < UB; ++u)
-            if (i0 + u < LDV) raw[u] = __ldg(col + i0 + u);
-            else raw[u] = make_int4(0, 0, 0, 0);
-#pragma unroll
-          for (int u = 0; u < UB; ++u) {
-            const int q = min(i0 + u, LDV - 1);
-            limb_fma(make_int2(raw[u].x, raw[u].y), tl[2 * q], h, m);
-            limb_fma(make_int2(raw[u].z, raw[u].w), tl[2 * q + 1], h, m);
-          }
-          carry(h, m);
-          hs += h >> 8;  // up to 254 rows
-          h &= 255;
-        }
-        y = fma((double)hs, 256.0, (double)h);
-        y = fma(y, (double)(1ll << kLimbBits), (double)m);
-        y = scale_pow2(y, scale_exp(all == kNone ? 1023 : all, (j % nt < nvel ? 0 : delta)));
-      } else {
-        const double* col = inv + (size_t)c * n * ld + (size_t)j * ld;
-        for (int i = 0; i < n; ++i) y = fma(col[i], td[i], y);
-      }
-      if (d_scatter) d_scatter[ic[j]] += omega * y;
-      else Y[(long long)c * n + j] = y;
-    }
-  }
-}
-
-template <int NR>
-stm_status launch_cells(const Level& L, const double* t, const int* cells, int nc, int ld, double* scatter, double omega,
+template <int K, int D>
+stm_status launch_cells(const Level& L, const double* t, const int* cells, int nc, double* scatter, double omega,
                         cudaStream_t s) {
-  static int per_sm = 0;
-  if (!per_sm) {
-    int o = 0;
-    STM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_limb_cells<NR>, 256, 0));
-    per_sm = std::max(o, 1);
-  }
-  // a warp per cell where that keeps every resident warp busy, more where cells are few
-  const long long most = 8LL * sm_count() * per_sm;
-  int G = 1;
-  while (G < 8 && nc * (long long)G * 2 <= most) G *= 2;
+  const int ld = inv_layout(Cell<K, D>::n, STM_F64).ld;
   // as few CTAs as give the same number of rounds, so that none idles through a last partial one
-  const long long ctas = ((long long)nc * G + 7) / 8, rounds = (ctas + most / 8 - 1) / (most / 8);
-  k_limb_cells<NR><<<(int)((ctas + rounds - 1) / rounds), 256, 0, s>>>(
-      (const int4*)L.lim, L.lexp, (const double*)L.inv, L.idx, t, L.Y, cells, nc, L.n, ld, G, L.nt, L.dim * L.nv, scatter, omega);
+  const int most = kCtas * sm_count(), ctas = (nc + 7) / 8, rounds = (ctas + most - 1) / most;
+  k_limb_cells<K, D><<<(ctas + rounds - 1) / rounds, 256, 0, s>>>((const int4*)L.lim, L.lexp, (const double*)L.inv, L.idx,
+                                                                  t, L.Y, cells, nc, ld, scatter, omega);
+  note_launch();
+  STM_CUDA(cudaGetLastError());
   return STM_OK;
 }
 
 }  // namespace
 
-stm_status inverse_limbs(Level& L, cudaStream_t s) {
-  const int ld = inv_layout(L.n, STM_F64).ld;
-  if (ld % 2 || L.n < 32 || L.n > 254) return STM_OK;
+bool limb_cells_pay(int nc) { return 5 * nc > 4 * 8 * kCtas * sm_count(); }
+
+// The elements whose cells have 32 rows and more and whose inverse is formed at all: 42 and 63 rows in 2D, 85 and 170 in 3D
+#define STM_CELLS(L, call)                          \
+  switch ((L).dim * 10 + (L).K) {                   \
+    case 22: { constexpr int K = 2, D = 2; call; break; } \
+    case 23: { constexpr int K = 3, D = 2; call; break; } \
+    case 31: { constexpr int K = 1, D = 3; call; break; } \
+    case 32: { constexpr int K = 2, D = 3; call; break; } \
+    default: break;                                 \
+  }
+
+stm_status inverse_limbs(Level& L, int nc, cudaStream_t s) {
+  const int ld = inv_layout(L.n, STM_F64).ld, nk = L.K * (L.dim + 1);
+  if (ld % 2 || L.n < 32 || L.n > 192 || !limb_cells_pay(nc)) return STM_OK;
   if (!L.lim) {
     // a second copy of the inverses: without room for it the FP64 kernels serve
     if (cudaMalloc((void**)&L.lim, sizeof(int2) * (size_t)L.C * L.n * ld) != cudaSuccess ||
-        cudaMalloc((void**)&L.lexp, sizeof(int) * (size_t)L.C * (L.n + 1)) != cudaSuccess) {
+        cudaMalloc((void**)&L.lexp, sizeof(short) * (size_t)L.C * nk * ld) != cudaSuccess) {
       cudaGetLastError();
       if (L.lim) cudaFree(L.lim);
       L.lim = nullptr;
       return STM_OK;
     }
   }
-  k_inverse_limbs<<<L.C, 256, 0, s>>>((const double*)L.inv, L.n, ld, L.nt, L.dim * L.nv, L.lim, L.lexp);
+  STM_CELLS(L, (k_inverse_limbs<K, D><<<L.C, 256, 0, s>>>((const double*)L.inv, ld, L.lim, L.lexp)));
   note_launch();
   STM_CUDA(cudaGetLastError());
   return STM_OK;
 }
 
-stm_status vanka_limbs(const Level& L, const double* t, const int* cells, int nc, int transpose, double* scatter,
-                       double omega, cudaStream_t s) {
-  const int n = L.n, ld = inv_layout(n, STM_F64).ld;
-  if (transpose) {
-    const int T = (n + 31) / 32 * 32, P = std::min(16, std::max(1, 256 / T));
-    const int blocks = std::min((nc + P - 1) / P, sm_count() * 8);
-    k_limb_cells_t<<<blocks, T * P, sizeof(int2) * (size_t)P * ld, s>>>((const int4*)L.lim, L.lexp, (const double*)L.inv,
-                                                                       L.idx, t, L.Y, cells, nc, n, ld, T, P, L.nt,
-                                                                       L.dim * L.nv, scatter, omega);
-  } else if (n <= 64) {
-    STM_TRY(launch_cells<1>(L, t, cells, nc, ld, scatter, omega, s));
-  } else if (n <= 128) {
-    STM_TRY(launch_cells<2>(L, t, cells, nc, ld, scatter, omega, s));
-  } else if (n <= 192) {
-    STM_TRY(launch_cells<3>(L, t, cells, nc, ld, scatter, omega, s));
-  } else {
-    STM_TRY(launch_cells<4>(L, t, cells, nc, ld, scatter, omega, s));
-  }
-  note_launch();
-  STM_CUDA(cudaGetLastError());
-  return STM_OK;
+stm_status vanka_limbs(const Level& L, const double* t, const int* cells, int nc, double* scatter, double omega,
+                       cudaStream_t s) {
+  STM_CELLS(L, return (launch_cells<K, D>(L, t, cells, nc, scatter, omega, s)));
+  set_error("cell solves over limbs: unsupported (dim, k)");
+  return STM_ERR_INVALID_ARG;
 }
 
 }  // namespace stm

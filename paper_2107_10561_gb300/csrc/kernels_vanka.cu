@@ -6,7 +6,7 @@
 // thread owns a fixed chunk of V consecutive rows and walks the columns with aligned 16/8/4-byte
 // vector loads: consecutive threads read consecutive memory, every load is fully used, no
 // per-element reductions. Small cells are packed several per CTA to keep enough loads in flight.
-// FP64 inverses of cells of 32 rows and more have kernels of their own (kernels_limb_vanka.cu).
+// Many cells of 32 rows and more with FP64 inverses have a kernel of their own (kernels_limb_vanka.cu).
 // Shared DoFs are combined in a second, deterministic pass:
 //   additive : d_i += omega / m_i * sum over the owners of i of y_T[alpha]
 //   overwrite: d_i += omega * y_Tlast[alpha] (highest-index owning cell, "last update wins")
@@ -418,7 +418,7 @@ static stm_status launch_local(Hierarchy& H, Level& L, int level, const double* 
   ProfScope ps(&H, STM_KCLASS_VANKA_LOCAL, s, (double)nc * ((double)L.n * L.n * storage_size(prec) + 20.0 * L.n),
                level);
   const double omega = H.p.omega;
-  if (prec == STM_F64 && L.lim) return vanka_limbs(L, t, cells, nc, transpose, scatter, omega, s);
+  if (prec == STM_F64 && L.lim && !transpose && limb_cells_pay(nc)) return vanka_limbs(L, t, cells, nc, scatter, omega, s);
   if (!transpose) {
     const VGeom g = vanka_geometry(L.n, lay, prec);
     if (prec == STM_F64) launch_fwd<double>(L, L.inv, lay.vb, g, t, cells, nc, scatter, omega, s);
