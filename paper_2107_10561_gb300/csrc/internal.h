@@ -237,16 +237,17 @@ struct Level {
   double *d = nullptr, *r = nullptr, *t = nullptr;
   // multi-right-hand-side work space ([N][32] interleaved; mY: [C*n][32]), allocated on first use
   double *md = nullptr, *mr = nullptr, *mt = nullptr, *mY = nullptr;
-  // the 32-column product's operands (kernels_digit_spmm.cu): steps of 16 positions of node i from dbase[i],
-  // the velocity rows of J and J^T in fragment order with a power of two per row, X's words and bases
+  // the 32-column product's operands (kernels_digit_spmm.cu): steps of 16 neighbours per component of node i from
+  // dbase[i], the velocity columns of J's and J^T's velocity rows in fragment order with a power of two per row and
+  // component, X's halves and bases
   int* dbase = nullptr;           // [R+1]
   long long dsteps = 0;
   void* jw[2] = {};
-  int* jwexp[2] = {};
+  int* jwexp[2] = {};             // [R][K*d components][K*d rows]
   bool jw_current[2] = {};        // built from the present values
   void* xw = nullptr;
   short *xb = nullptr, *xnb = nullptr;  // bases of X, and the largest ones around every node
-  void* xmost = nullptr;
+  void *xcb = nullptr, *xmost = nullptr;  // largest and smallest ones of every cell; largest shifts around every node
   uint32_t* mt16 = nullptr;       // [N][32] the smoothing step's residual block as packed BF16 (lo << 16 | hi)
 };
 

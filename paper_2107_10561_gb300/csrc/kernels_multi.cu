@@ -1,8 +1,8 @@
 // Multi-right-hand-side path: up to 32 right-hand sides share one hierarchy (one J, one set of
 // cell inverses). Multi-vectors are stored interleaved, [N][32] FP64 (column c of DoF i at
 // i * 32 + c), so every gather of a DoF fetches its 32 values in one 256-byte line.
-//  * SpMM with J_g: on the tensor cores over base-256 digits (kernels_digit_spmm.cu); with more than six
-//    velocity rows per node (3D dG(2)) here in FP64, one warp per node (cell) with the 32 lanes on the
+//  * SpMM with J_g: with six velocity rows per node (3D dG(1), 2D dG(2)) on the tensor cores over base-256
+//    digits (kernels_digit_spmm.cu); else here in FP64, one warp per node (cell) with the 32 lanes on the
 //    32 right-hand sides: each value of J is read once for all columns (broadcast).
 //  * Vanka local solves Y_T = J_T^{-1} T_T for a 32-column block (a6'' of the hot path): with BF16
 //    inverses on the tcgen05 tensor cores (kernels_mrhs_tc.cu: TMA-staged inverses, FP32 accumulators
@@ -206,7 +206,9 @@ stm_status spmm_structured(Level& L, const double* X, const double* B, double* Y
   k_spmm_struct<K, D><<<blocks, 256, 0, s>>>(L.rowptr, L.val, L.nbr_ptr, L.nbr, L.ncell, L.node_cells, L.cell_nodes, \
                                              L.block, L.R, L.C, L.nv, X, B, Y, mode, L.valT, split, T16)
   switch (key) {
-    case 33: SPMM(3, 3); break;  // nine rows per node
+    case 21: SPMM(1, 2); break;
+    case 22: SPMM(2, 2); break;
+    case 31: SPMM(1, 3); break;
     default:
       set_error("multi-RHS SpMM: unsupported (dim, k)");
       return STM_ERR_INVALID_ARG;
