@@ -437,7 +437,8 @@ __global__ void __launch_bounds__(256) k_gj_panel(double* __restrict__ A, int n,
       }
       break;
     }
-    if (rank == 0 && tid == 0) piv[gk] = p;
+    // after a wait that ran out the row may be anything: what follows indexes with it
+    if (rank == 0 && tid == 0) piv[gk] = p >= gk && p < n ? p : gk;
     const double* prow = box + (size_t)who * wp;
     const double* krow = box + (size_t)NC * wp;
     const double pinv = cand[2 * who + 1];
