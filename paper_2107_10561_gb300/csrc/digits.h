@@ -115,14 +115,5 @@ __device__ __forceinline__ long long abs_key(double v) {
   const long long k = __double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll;
   return k > 0x7FF0000000000000ll ? -1 : k;
 }
-// 1 / a: the hardware's approximation and two Newton steps, four dependent FP64 operations
-__device__ __forceinline__ double reciprocal(double a) {
-  const int ex = (__double2hiint(a) >> 20) & 0x7FF;
-  if (ex < 64 || ex > 1982) return 1.0 / a;
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-  r = fma(r, fma(-a, r, 1.0), r);
-  return fma(r, fma(-a, r, 1.0), r);
-}
 
 }  // namespace stm

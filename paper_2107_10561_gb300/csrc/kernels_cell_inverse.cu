@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_cell_inverse(const
           if (bk <= 0 || bk >= 0x7FF0000000000000ll) {
             if (lane == 0) s_bad = 1;
           } else {
-            const double pr = P[bi * kPitch + j16], inv1 = reciprocal(P[bi * kPitch + k]);
+            const double pr = P[bi * kPitch + j16], inv1 = 1.0 / P[bi * kPitch + k];
             if (lane < kPanel) {
               kbuf[lane] = P[gk * kPitch + lane];
               ubuf[lane] = lane == k ? inv1 : pr * inv1;

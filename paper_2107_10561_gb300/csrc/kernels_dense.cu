@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(256) k_gj_panel(double* __restrict__ A, int n,
       bi = __shfl_sync(0xffffffffu, row, l);
     }
     if (warp == 7) {  // the reciprocal takes longest
-      const double inv = bk >= 0 ? reciprocal(P[(size_t)(bi - r0) * ws + k]) : 0.0;
+      const double inv = bk >= 0 ? 1.0 / P[(size_t)(bi - r0) * ws + k] : 0.0;
       const uint32_t at = smem_addr(box + (size_t)(NC + 1) * wp + 2 * rank);
       if (lane < NC) remote_store(at, bar, lane, __longlong_as_double(bk), inv);
       else if (lane < 2 * NC) remote_store(at + 16 * NC, bar, lane - NC, __longlong_as_double(bi), 0.0);
