@@ -240,17 +240,17 @@ __global__ void k_scale_host(double* y, const double* x, double f, long long n) 
 
 static stm_status ensure_krylov(Hierarchy& H, int m) {
   const long long N = H.L.back().N;
-  if (H.restart_cap >= m && H.V) return STM_OK;
-  void* ptrs[] = {H.V, H.Z, H.w, H.hcol, H.part, H.yvec};
-  for (void* q : ptrs)
-    if (q) cudaFree(q);
+  if (H.restart_cap >= m) return STM_OK;
+  double** ptrs[] = {&H.V, &H.Z, &H.w, &H.hcol, &H.part, &H.yvec};
   H.nblk_dot = 304;
-  STM_CUDA(cudaMalloc(&H.V, sizeof(double) * (size_t)(m + 1) * N));
-  STM_CUDA(cudaMalloc(&H.Z, sizeof(double) * (size_t)m * N));
-  STM_CUDA(cudaMalloc(&H.w, sizeof(double) * (size_t)N));
-  STM_CUDA(cudaMalloc(&H.hcol, sizeof(double) * (size_t)(2 * m + 8)));
-  STM_CUDA(cudaMalloc(&H.part, sizeof(double) * (size_t)(m + 2) * H.nblk_dot));
-  STM_CUDA(cudaMalloc(&H.yvec, sizeof(double) * (size_t)(m + 2)));
+  const size_t len[] = {(size_t)(m + 1) * N, (size_t)m * N, (size_t)N, (size_t)(2 * m + 8), (size_t)(m + 2) * H.nblk_dot,
+                        (size_t)(m + 2)};
+  for (double** q : ptrs) {
+    if (*q) cudaFree(*q);
+    *q = nullptr;
+  }
+  H.restart_cap = 0;
+  for (int i = 0; i < 6; ++i) STM_TRY(device_alloc(H, ptrs[i], sizeof(double) * len[i]));
   H.restart_cap = m;
   return STM_OK;
 }
@@ -424,8 +424,8 @@ stm_status stm_gmres_solve_host(stm_hierarchy* h, const double* b_host, double* 
   Hierarchy& H = h->H;
   const long long N = H.L.back().N;
   cudaStream_t s = S(stream);
-  if (!H.bbuf) STM_CUDA(cudaMalloc(&H.bbuf, sizeof(double) * N));
-  if (!H.xbuf) STM_CUDA(cudaMalloc(&H.xbuf, sizeof(double) * N));
+  if (!H.bbuf) STM_TRY(device_alloc(H, &H.bbuf, sizeof(double) * N));
+  if (!H.xbuf) STM_TRY(device_alloc(H, &H.xbuf, sizeof(double) * N));
   STM_CUDA(cudaMemcpyAsync(H.bbuf, b_host, sizeof(double) * N, cudaMemcpyHostToDevice, s));
   if (opts->use_x0) STM_CUDA(cudaMemcpyAsync(H.xbuf, x_host, sizeof(double) * N, cudaMemcpyHostToDevice, s));
   stm_status st = stm_gmres_solve(h, H.bbuf, H.xbuf, opts, info, stream);
@@ -481,7 +481,7 @@ stm_status stm_newton_solve(stm_hierarchy* h, double U, double nu, double* X, co
   STM_TRY(ensure_krylov(H, gopts->restart));
   double** bufs[] = {&H.nw_negF, &H.nw_D, &H.nw_Xt, &H.nw_B, &H.nw_Ft};
   for (double** b : bufs)
-    if (!*b) STM_CUDA(cudaMalloc((void**)b, sizeof(double) * N));
+    if (!*b) STM_TRY(device_alloc(H, b, sizeof(double) * N));
   // the previous slab's last time node (right Radau: the slab end) carries v(t_{n-1}^-)
   const double* vprev = prev ? prev + (long long)(H.L.back().K - 1) * H.L.back().block : nullptr;
   stm_newton_info inf{};
@@ -558,7 +558,7 @@ stm_status stm_assemble_load(stm_hierarchy* h, double U, double nu, const double
     return assemble_cellvec(H, 0, U, nu, nullptr, nullptr, b_dev, s);
   }
   const Level& F = H.L.back();
-  if (!H.ag_wnod) STM_CUDA(cudaMalloc(&H.ag_wnod, sizeof(double) * (size_t)F.K * F.dim * F.R));
+  if (!H.ag_wnod) STM_TRY(device_alloc(H, &H.ag_wnod, sizeof(double) * (size_t)F.K * F.dim * F.R));
   STM_TRY(inject_level(H, (int)H.L.size() - 1, w_dev, H.ag_wnod, s));
   return assemble_cellvec(H, 0, U, nu, nullptr, nullptr, b_dev, s, nullptr, H.ag_wnod);
 }
@@ -576,7 +576,7 @@ stm_status stm_adjoint_gradient(stm_hierarchy* h, double U, double nu, const dou
   }
   const long long N = H.L.back().N;
   cudaStream_t s = S(stream);
-  if (!H.ag_buf) STM_CUDA(cudaMalloc(&H.ag_buf, sizeof(double) * 4 * (size_t)N));
+  if (!H.ag_buf) STM_TRY(device_alloc(H, &H.ag_buf, sizeof(double) * 4 * (size_t)N));
   double* dbdU = H.ag_buf;  // db/dU, db/dnu and (dJ/dnu) X back to back: one batched dot with lambda
   double* dbdnu = dbdU + N;
   double* dJX = dbdnu + N;
@@ -681,19 +681,15 @@ stm_status stm_vanka_sweep_fused(stm_hierarchy* h, int level, int n_fwd, const d
 
 static stm_status ensure_krylov_multi(Hierarchy& H, int m) {
   const size_t N = (size_t)H.L.back().N, NRs = 32;
-  if (H.mrestart_cap >= m && H.mV) return STM_OK;
-  void* ptrs[] = {H.mV, H.mZ, H.mW, H.mB, H.mX, H.mh, H.mpart, H.mf, H.my};
-  for (void* q : ptrs)
-    if (q) cudaFree(q);
-  STM_CUDA(cudaMalloc(&H.mV, sizeof(double) * (m + 1) * N * NRs));
-  STM_CUDA(cudaMalloc(&H.mZ, sizeof(double) * m * N * NRs));
-  STM_CUDA(cudaMalloc(&H.mW, sizeof(double) * N * NRs));
-  STM_CUDA(cudaMalloc(&H.mB, sizeof(double) * N * NRs));
-  STM_CUDA(cudaMalloc(&H.mX, sizeof(double) * N * NRs));
-  STM_CUDA(cudaMalloc(&H.mh, sizeof(double) * (2 * m + 8) * NRs));
-  STM_CUDA(cudaMalloc(&H.mpart, sizeof(double) * (m + 2) * 304 * NRs));
-  STM_CUDA(cudaMalloc(&H.mf, sizeof(double) * NRs));
-  STM_CUDA(cudaMalloc(&H.my, sizeof(double) * (m + 1) * NRs));
+  if (H.mrestart_cap >= m) return STM_OK;
+  double** ptrs[] = {&H.mV, &H.mZ, &H.mW, &H.mB, &H.mX, &H.mh, &H.mpart, &H.mf, &H.my};
+  const size_t len[] = {(m + 1) * N, m * N, N, N, N, (size_t)(2 * m + 8), (size_t)(m + 2) * 304, 1, (size_t)(m + 1)};
+  for (double** q : ptrs) {
+    if (*q) cudaFree(*q);
+    *q = nullptr;
+  }
+  H.mrestart_cap = 0;
+  for (int i = 0; i < 9; ++i) STM_TRY(device_alloc(H, ptrs[i], sizeof(double) * len[i] * NRs));
   H.mrestart_cap = m;
   return STM_OK;
 }

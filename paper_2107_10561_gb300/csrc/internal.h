@@ -210,6 +210,8 @@ struct Level {
   void* inv = nullptr;            // [C][n*n] column-major per cell, storage precision
   int2* lim = nullptr;            // FP64 inverses once more as two-limb integers, same layout (null: no room)
   short* lexp = nullptr;          // [C][classes of columns][ld] the exponents of their rows by class
+  bool lim_current = false;       // built from the present inverses
+  bool lim_off = false;           // no room for them until the next factorisation
   double* wmult = nullptr;        // [N] 1/m_i
   int* own_ptr = nullptr;         // [N+1]
   int* own_pos = nullptr;         // [sum m_i] flat positions c*n + alpha
@@ -245,6 +247,7 @@ struct Level {
   void* jw[2] = {};
   int* jwexp[2] = {};             // [R][K*d components][K*d rows]
   bool jw_current[2] = {};        // built from the present values
+  bool digits_off = false;        // no room for these operands: the product runs in FP64
   void* xw = nullptr;
   short *xb = nullptr, *xnb = nullptr;  // bases of X, and the largest ones around every node
   void *xcb = nullptr, *xmost = nullptr;  // largest and smallest ones of every cell; largest shifts around every node
@@ -356,11 +359,20 @@ stm_status launch_fill_colidx(Level& Lv, const int* nbr_ptr, const int* nbr_idx,
 stm_status inject_linearisation(Hierarchy& H, const double* X_fine, cudaStream_t s);
 stm_status assemble_level(Hierarchy& H, int g, double nu, cudaStream_t s);
 stm_status factor_level(Hierarchy& H, int g, cudaStream_t s);
-// FP64 inverses: their copy in limbs and the cell solves with it (kernels_limb_vanka.cu), for nc cells at a time
+// FP64 inverses: their copy in limbs, made before the first cell solves that gain from it where there is room, and the cell
+// solves with it (kernels_limb_vanka.cu)
 bool limb_cells_pay(int nc);
-stm_status inverse_limbs(Level& L, int nc, cudaStream_t s);
+stm_status ensure_inverse_limbs(Hierarchy& H, int g, cudaStream_t s);
+void free_inverse_limbs(Level& L);
 stm_status vanka_limbs(const Level& L, const double* t, const int* cells, int nc, double* scatter, double omega,
                        cudaStream_t s);
+// Device memory that a call cannot do without: where it does not fit, what only saves time is given back first (copies of
+// the inverses, operands of the 32-column product, the coarse factorisation's work space; graphs that use them).
+stm_status device_alloc(Hierarchy& H, void** p, size_t bytes);
+void give_back(Hierarchy& H);
+template <typename T>
+stm_status device_alloc(Hierarchy& H, T** p, size_t bytes) { return device_alloc(H, (void**)p, bytes); }
+void free_spmm_digits(Level& L);
 stm_status factor_coarse(Hierarchy& H, cudaStream_t s);
 stm_status ensure_transpose(Hierarchy& H, int g, cudaStream_t s);
 // Dense FP64 products and inverses on the tensor cores (kernels_dense.cu). An operand is cut into digits in

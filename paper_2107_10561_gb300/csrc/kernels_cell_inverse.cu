@@ -409,7 +409,7 @@ stm_status factor_level(Hierarchy& H, int g, cudaStream_t s) {
   Level& L = H.L[g];
   const int n = L.n;
   const InvLayout lay = inv_layout(n, H.p.inv_precision);
-  if (!L.inv) STM_CUDA(cudaMalloc(&L.inv, storage_bytes(H.p.inv_precision) * (size_t)n * lay.ld * L.C));
+  if (!L.inv) STM_TRY(device_alloc(H, &L.inv, storage_bytes(H.p.inv_precision) * (size_t)n * lay.ld * L.C));
   int dev = 0, maxsm = 0;
   STM_CUDA(cudaGetDevice(&dev));
   STM_CUDA(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
@@ -428,16 +428,15 @@ stm_status factor_level(Hierarchy& H, int g, cudaStream_t s) {
     if (H.cell_scratch) cudaFree(H.cell_scratch);
     H.cell_scratch = nullptr;
     H.cell_scratch_len = 0;
-    STM_CUDA(cudaMalloc(&H.cell_scratch, sizeof(double) * (size_t)blocks * n * n));
+    STM_TRY(device_alloc(H, &H.cell_scratch, sizeof(double) * (size_t)blocks * n * n));
     H.cell_scratch_len = (long long)blocks * n * n;
   }
   const size_t smem = cell_smem(n, in_smem).total;
   a.scratch = in_smem ? nullptr : H.cell_scratch;
   if (per_sm == 4) STM_TRY(launch<128>(H, a, L.inv, blocks, smem, s));
   else STM_TRY(launch<256>(H, a, L.inv, blocks, smem, s));
-  // the coloured smoother solves on the cells of one colour at a time
-  const int nc = H.p.smoother == STM_VANKA_COLOURED ? L.C >> L.dim : L.C;
-  return H.p.inv_precision == STM_F64 ? inverse_limbs(L, nc, s) : STM_OK;
+  L.lim_current = L.lim_off = false;
+  return STM_OK;
 }
 
 }  // namespace stm

@@ -571,11 +571,13 @@ stm_status coarse_slab_apply(Hierarchy& H, const double* r, double* d, int trans
 
 stm_status coarse_slab_apply_multi(Hierarchy& H, const double* R, double* D, cudaStream_t s) {
   const long long stride = (long long)groups_of(H.cs_maxnb, kChunk) * groups_of(H.cs_maxnb, 16) * 16 * NR;
-  if (!H.cs_mu) {
-    STM_CUDA(cudaMalloc(&H.cs_mu, sizeof(double) * 32 * (size_t)H.N0));
-    STM_CUDA(cudaMalloc(&H.cs_mv, sizeof(double) * 32 * (size_t)H.N0));
+  if (!H.cs_mu || !H.cs_mv) {
+    cudaFree(H.cs_mu);
+    H.cs_mu = nullptr;
+    STM_TRY(device_alloc(H, &H.cs_mu, sizeof(double) * 32 * (size_t)H.N0));
+    STM_TRY(device_alloc(H, &H.cs_mv, sizeof(double) * 32 * (size_t)H.N0));
   }
-  if (!H.cs_part) STM_CUDA(cudaMalloc(&H.cs_part, sizeof(double) * std::max(2, std::min(kBatch, H.cs_nx)) * (size_t)stride));
+  if (!H.cs_part) STM_TRY(device_alloc(H, &H.cs_part, sizeof(double) * std::max(2, std::min(kBatch, H.cs_nx)) * (size_t)stride));
   return launch_cooperative(k_coarse_slab_multi, 256, 1, s, view_of(H), R, D, H.cs_mu, H.cs_mv, H.cs_part, stride);
 }
 

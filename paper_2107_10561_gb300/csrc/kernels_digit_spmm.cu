@@ -483,7 +483,17 @@ stm_status launch(const Level& L, SpmmArgs& a, cudaStream_t s) {
 // 361, dG(0), 45,698: 106 against 221; 3D dG(0), 64,547: 708 against 725).
 bool spmm_digits_supported(const Level& L) { return L.K * L.dim == 6; }
 
-// J's words (and J^T's when transpose is set) for the present values; work space on first use
+void free_spmm_digits(Level& L) {
+  void* ptrs[] = {L.xw, L.xb, L.xcb, L.xnb, L.xmost, L.jw[0], L.jw[1], L.jwexp[0], L.jwexp[1]};
+  for (void* q : ptrs) cudaFree(q);
+  L.xw = L.xcb = L.xmost = L.jw[0] = L.jw[1] = nullptr;
+  L.xb = L.xnb = nullptr;
+  L.jwexp[0] = L.jwexp[1] = nullptr;
+  L.jw_current[0] = L.jw_current[1] = false;
+}
+
+// J's words (and J^T's when transpose is set) for the present values; work space on first use. STM_ERR_OOM where it
+// does not fit, and nothing is kept then.
 stm_status ensure_spmm_digits(Level& L, int transpose, cudaStream_t s) {
   const int KD = L.K * L.dim;
   if (!L.dbase) {
@@ -495,14 +505,21 @@ stm_status ensure_spmm_digits(Level& L, int transpose, cudaStream_t s) {
     STM_CUDA(cudaMemcpy(L.dbase, dbase.data(), sizeof(int) * (L.R + 1), cudaMemcpyHostToDevice));
     L.dsteps = dbase[L.R];
   }
-  if (!L.xw) STM_CUDA(cudaMalloc(&L.xw, sizeof(uint2) * NR * KD * (size_t)L.R));
-  if (!L.xb) STM_CUDA(cudaMalloc((void**)&L.xb, sizeof(short) * NR * KD * (size_t)L.R));
-  if (!L.xcb) STM_CUDA(cudaMalloc(&L.xcb, sizeof(short2) * NR * KD * (size_t)L.C));
-  if (!L.xnb) STM_CUDA(cudaMalloc((void**)&L.xnb, sizeof(short) * NR * KD * (size_t)L.R));
-  if (!L.xmost) STM_CUDA(cudaMalloc(&L.xmost, 16 * (size_t)L.R));
+  struct { void** p; size_t bytes; } want[] = {
+      {&L.xw, sizeof(uint2) * NR * KD * (size_t)L.R}, {(void**)&L.xb, sizeof(short) * NR * KD * (size_t)L.R},
+      {&L.xcb, sizeof(short2) * NR * KD * (size_t)L.C}, {(void**)&L.xnb, sizeof(short) * NR * KD * (size_t)L.R},
+      {&L.xmost, 16 * (size_t)L.R}, {&L.jw[0], sizeof(uint4) * 8 * KD * (size_t)L.dsteps},
+      {(void**)&L.jwexp[0], sizeof(int) * KD * KD * (size_t)L.R}, {&L.jw[1], sizeof(uint4) * 8 * KD * (size_t)L.dsteps},
+      {(void**)&L.jwexp[1], sizeof(int) * KD * KD * (size_t)L.R}};
+  for (int i = 0; i < (transpose ? 9 : 7); ++i)
+    if (!*want[i].p && cudaMalloc(want[i].p, want[i].bytes) != cudaSuccess) {
+      cudaGetLastError();
+      *want[i].p = nullptr;
+      STM_CUDA(cudaStreamSynchronize(s));  // products that still read them
+      free_spmm_digits(L);
+      return STM_ERR_OOM;
+    }
   for (int t = 0; t <= (transpose ? 1 : 0); ++t) {
-    if (!L.jw[t]) STM_CUDA(cudaMalloc(&L.jw[t], sizeof(uint4) * 8 * KD * (size_t)L.dsteps));
-    if (!L.jwexp[t]) STM_CUDA(cudaMalloc((void**)&L.jwexp[t], sizeof(int) * KD * KD * (size_t)L.R));
     if (L.jw_current[t]) continue;
     const double* val = t ? L.valT : L.val;
     switch (L.dim * 10 + L.K) {

@@ -382,7 +382,16 @@ static stm_status twisted_slab_factors(Hierarchy& H, const Level& L, const std::
   return STM_OK;
 }
 
+static stm_status factor_coarse_in(Hierarchy& H, cudaStream_t s);
 stm_status factor_coarse(Hierarchy& H, cudaStream_t s) {
+  stm_status st = factor_coarse_in(H, s);
+  if (st == STM_ERR_OOM) {  // once more without what only saves time
+    give_back(H);
+    st = factor_coarse_in(H, s);
+  }
+  return st;
+}
+static stm_status factor_coarse_in(Hierarchy& H, cudaStream_t s) {
   Level& L = H.L[0];
   const long long n = L.N;
   const int nx = L.cells[0];

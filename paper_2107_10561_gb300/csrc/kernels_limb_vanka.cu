@@ -20,7 +20,7 @@
 //     cell (3D dG(1), 1,536 cells, whole sweep: 185 against 168 us; with several warps here 360 cells took 46 us against
 //     31), and so does the transpose (2D dG(2): 204 us against 145; the scales of its products differ from row to row of
 //     the inverse and class of columns). So do cells of fewer than 32 rows (2D dG(0): 21) and levels without
-//     room for the second copy.
+//     room for the second copy, which is made on the first solve and given back when memory runs short.
 //   - Cells with an infinity or a NaN, in the inverse or in t, are summed in FP64 from the FP64 inverses.
 #include "digits.h"
 #include "internal.h"
@@ -284,22 +284,45 @@ bool limb_cells_pay(int nc) { return 5 * nc > 4 * 8 * kCtas * sm_count(); }
     default: break;                                 \
   }
 
-stm_status inverse_limbs(Level& L, int nc, cudaStream_t s) {
+void free_inverse_limbs(Level& L) {
+  cudaFree(L.lim);
+  cudaFree(L.lexp);
+  L.lim = nullptr;
+  L.lexp = nullptr;
+  L.lim_current = false;
+}
+
+// A second copy of the inverses, on the first cell solve after a factorisation. Where it would not leave room for the
+// Krylov basis, J^T and something for others the FP64 kernels serve.
+stm_status ensure_inverse_limbs(Hierarchy& H, int g, cudaStream_t s) {
+  Level& L = H.L[g];
+  if (H.p.inv_precision != STM_F64 || L.lim_current || L.lim_off || !L.inv) return STM_OK;
   const int ld = inv_layout(L.n, STM_F64).ld, nk = L.K * (L.dim + 1);
+  // the coloured smoother solves on the cells of one colour at a time
+  const int nc = H.p.smoother == STM_VANKA_COLOURED ? L.C >> L.dim : L.C;
   if (ld % 2 || L.n < 32 || L.n > 192 || !limb_cells_pay(nc)) return STM_OK;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  STM_CUDA(cudaStreamIsCapturing(s, &capture));
+  if (capture != cudaStreamCaptureStatusNone) return STM_OK;
   if (!L.lim) {
-    // a second copy of the inverses: without room for it the FP64 kernels serve
-    if (cudaMalloc((void**)&L.lim, sizeof(int2) * (size_t)L.C * L.n * ld) != cudaSuccess ||
-        cudaMalloc((void**)&L.lexp, sizeof(short) * (size_t)L.C * nk * ld) != cudaSuccess) {
+    const size_t limbs = sizeof(int2) * (size_t)L.C * L.n * ld, exps = sizeof(short) * (size_t)L.C * nk * ld;
+    size_t room = 0, all = 0, later = (size_t)2 << 30;
+    if (!H.V) later += sizeof(double) * 62 * (size_t)H.L.back().N;
+    for (const Level& l : H.L)
+      if (!l.valT) later += sizeof(double) * (size_t)(l.nnz + l.nval_cap + l.pval_len);
+    STM_CUDA(cudaMemGetInfo(&room, &all));
+    if (room < limbs + exps + later || cudaMalloc((void**)&L.lim, limbs) != cudaSuccess ||
+        cudaMalloc((void**)&L.lexp, exps) != cudaSuccess) {
       cudaGetLastError();
-      if (L.lim) cudaFree(L.lim);
-      L.lim = nullptr;
+      free_inverse_limbs(L);
+      L.lim_off = true;
       return STM_OK;
     }
   }
   STM_CELLS(L, (k_inverse_limbs<K, D><<<L.C, 256, 0, s>>>((const double*)L.inv, ld, L.lim, L.lexp)));
   note_launch();
   STM_CUDA(cudaGetLastError());
+  L.lim_current = true;
   return STM_OK;
 }
 

@@ -93,10 +93,52 @@ __global__ void k_transpose_values(const long long* __restrict__ rowptr, const i
   }
 }
 
+// What a later call can do without, only slower, and work space between two factorisations. Work that uses it may still
+// be under way.
+void give_back(Hierarchy& H) {
+  cudaDeviceSynchronize();
+  clear_graphs(H);
+  for (Level& L : H.L) {
+    free_inverse_limbs(L);
+    L.lim_off = true;
+    free_spmm_digits(L);
+    L.digits_off = true;
+  }
+  for (DenseWork& w : H.dw) dense_free(w);
+  cudaFree(H.cs_raw);
+  cudaFree(H.cs_store);  // the solves read cs_words
+  H.cs_raw = H.cs_store = nullptr;
+}
+
+stm_status device_alloc(Hierarchy& H, void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    give_back(H);
+    e = cudaMalloc(p, bytes);
+  }
+  if (e == cudaSuccess) return STM_OK;
+  *p = nullptr;
+  return cuda_fail(e, "cudaMalloc");
+}
+
+static stm_status transpose_copies(Hierarchy& H, int g, cudaStream_t s);
 stm_status ensure_transpose(Hierarchy& H, int g, cudaStream_t s) {
   Level& L = H.L[g];
   if (L.valT) return STM_OK;
-  STM_CUDA(cudaMalloc(&L.valT, sizeof(double) * L.nnz));
+  const stm_status st = transpose_copies(H, g, s);
+  if (st != STM_OK) {  // none of it, so that the next call starts over
+    cudaStreamSynchronize(s);
+    void* ptrs[] = {L.valT, L.nvalJT, L.pvalJT, L.nexpJT};
+    for (void* q : ptrs) cudaFree(q);
+    L.valT = L.nvalJT = L.pvalJT = nullptr;
+    L.nexpJT = nullptr;
+  }
+  return st;
+}
+static stm_status transpose_copies(Hierarchy& H, int g, cudaStream_t s) {
+  Level& L = H.L[g];
+  STM_TRY(device_alloc(H, &L.valT, sizeof(double) * L.nnz));
   STM_CUDA(cudaMemsetAsync(H.dflag + 2, 0, sizeof(int), s));
   const int blocks = (int)std::min<long long>((L.N + 7) / 8, (long long)sms() * 16);
   k_transpose_values<<<blocks, 256, 0, s>>>(L.rowptr, L.colidx, L.val, L.valT, L.N, H.dflag + 2); note_launch();
@@ -109,10 +151,10 @@ stm_status ensure_transpose(Hierarchy& H, int g, cudaStream_t s) {
     return STM_ERR_STATE;
   }
   // node-block and pressure-row copies of J^T for the transposed SpMV
-  STM_CUDA(cudaMalloc(&L.nvalJT, sizeof(double) * L.nval_cap));
-  STM_CUDA(cudaMalloc(&L.pvalJT, sizeof(double) * L.pval_len));
+  STM_TRY(device_alloc(H, &L.nvalJT, sizeof(double) * L.nval_cap));
+  STM_TRY(device_alloc(H, &L.pvalJT, sizeof(double) * L.pval_len));
   STM_CUDA(cudaMemsetAsync(L.pvalJT, 0, sizeof(double) * L.pval_len, s));
-  if (L.limb_lanes) STM_CUDA(cudaMalloc(&L.nexpJT, limb_node_exps(L)));
+  if (L.limb_lanes) STM_TRY(device_alloc(H, &L.nexpJT, limb_node_exps(L)));
   STM_TRY(build_nodeblock(L, 1, s));
   if (H.p.defect_precision == STM_F32) STM_TRY(build_values_f32(L, 1, s));
   return STM_OK;
@@ -241,8 +283,10 @@ stm_status vcycle_graph(Hierarchy& H, const double* r, double* d, int transpose,
   const auto key = std::make_tuple(r, d, transpose);
   auto it = H.vgraphs.find(key);
   if (it == H.vgraphs.end()) {
-    if (transpose)
-      for (int g = 0; g < (int)H.L.size(); ++g) STM_TRY(ensure_transpose(H, g, s));
+    for (int g = 0; g < (int)H.L.size(); ++g) {
+      if (transpose) STM_TRY(ensure_transpose(H, g, s));
+      else if (g > 0) STM_TRY(ensure_inverse_limbs(H, g, s));
+    }
     if (!H.cap_stream) STM_CUDA(cudaStreamCreateWithFlags(&H.cap_stream, cudaStreamNonBlocking));
     const long long before = g_launches.load();
     STM_CUDA(cudaStreamBeginCapture(H.cap_stream, cudaStreamCaptureModeThreadLocal));

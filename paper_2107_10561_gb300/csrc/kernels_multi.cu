@@ -2,7 +2,7 @@
 // cell inverses). Multi-vectors are stored interleaved, [N][32] FP64 (column c of DoF i at
 // i * 32 + c), so every gather of a DoF fetches its 32 values in one 256-byte line.
 //  * SpMM with J_g: with six velocity rows per node (3D dG(1), 2D dG(2)) on the tensor cores over base-256
-//    digits (kernels_digit_spmm.cu); else here in FP64, one warp per node (cell) with the 32 lanes on the
+//    digits (kernels_digit_spmm.cu) where there is room for them; else here in FP64, one warp per node (cell) with the 32 lanes on the
 //    32 right-hand sides: each value of J is read once for all columns (broadcast).
 //  * Vanka local solves Y_T = J_T^{-1} T_T for a 32-column block (a6'' of the hot path): with BF16
 //    inverses on the tcgen05 tensor cores (kernels_mrhs_tc.cu: TMA-staged inverses, FP32 accumulators
@@ -198,7 +198,11 @@ stm_status spmm_structured(Level& L, const double* X, const double* B, double* Y
     set_error("multi-RHS SpMM: the values of J^T are not built");
     return STM_ERR_STATE;
   }
-  if (spmm_digits_supported(L)) return spmm_digits(L, X, B, Y, mode, s, split, T16);
+  if (spmm_digits_supported(L) && !L.digits_off) {
+    const stm_status st = spmm_digits(L, X, B, Y, mode, s, split, T16);
+    if (st != STM_ERR_OOM) return st;
+    L.digits_off = true;  // no room for its operands
+  }
   const long long jobs = (long long)L.R + L.C;
   const int blocks = (int)std::min<long long>((jobs * 32 + 255) / 256, (long long)msms() * 8);
   const int key = L.dim * 10 + L.K;
@@ -208,7 +212,9 @@ stm_status spmm_structured(Level& L, const double* X, const double* B, double* Y
   switch (key) {
     case 21: SPMM(1, 2); break;
     case 22: SPMM(2, 2); break;
+    case 23: SPMM(3, 2); break;
     case 31: SPMM(1, 3); break;
+    case 32: SPMM(2, 3); break;
     default:
       set_error("multi-RHS SpMM: unsupported (dim, k)");
       return STM_ERR_INVALID_ARG;
@@ -306,14 +312,10 @@ __global__ void k_vanka_gather_multi(double* __restrict__ d, const A* __restrict
 
 stm_status ensure_multi(Hierarchy& H) {
   for (Level& L : H.L) {
-    if (L.mY && L.md && (L.mt16 || H.p.inv_precision != STM_BF16)) continue;
-    if (!L.md) {
-      STM_CUDA(cudaMalloc(&L.md, sizeof(double) * (size_t)L.N * NR));
-      STM_CUDA(cudaMalloc(&L.mr, sizeof(double) * (size_t)L.N * NR));
-      STM_CUDA(cudaMalloc(&L.mt, sizeof(double) * (size_t)L.N * NR));
-    }
-    if (!L.mY) STM_CUDA(cudaMalloc(&L.mY, sizeof(double) * (size_t)L.C * L.n * NR));
-    if (!L.mt16 && H.p.inv_precision == STM_BF16) STM_CUDA(cudaMalloc(&L.mt16, sizeof(uint32_t) * (size_t)L.N * NR));
+    for (double** q : {&L.md, &L.mr, &L.mt})
+      if (!*q) STM_TRY(device_alloc(H, q, sizeof(double) * (size_t)L.N * NR));
+    if (!L.mY) STM_TRY(device_alloc(H, &L.mY, sizeof(double) * (size_t)L.C * L.n * NR));
+    if (!L.mt16 && H.p.inv_precision == STM_BF16) STM_TRY(device_alloc(H, &L.mt16, sizeof(uint32_t) * (size_t)L.N * NR));
   }
   return STM_OK;
 }

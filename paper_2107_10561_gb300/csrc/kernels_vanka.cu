@@ -418,7 +418,7 @@ static stm_status launch_local(Hierarchy& H, Level& L, int level, const double* 
   ProfScope ps(&H, STM_KCLASS_VANKA_LOCAL, s, (double)nc * ((double)L.n * L.n * storage_size(prec) + 20.0 * L.n),
                level);
   const double omega = H.p.omega;
-  if (prec == STM_F64 && L.lim && !transpose && limb_cells_pay(nc)) return vanka_limbs(L, t, cells, nc, scatter, omega, s);
+  if (prec == STM_F64 && L.lim_current && !transpose && limb_cells_pay(nc)) return vanka_limbs(L, t, cells, nc, scatter, omega, s);
   if (!transpose) {
     const VGeom g = vanka_geometry(L.n, lay, prec);
     if (prec == STM_F64) launch_fwd<double>(L, L.inv, lay.vb, g, t, cells, nc, scatter, omega, s);
@@ -470,6 +470,7 @@ stm_status vanka_step(Hierarchy& H, int g, const double* r, double* d, int trans
                       cudaStream_t s, bool d32_current) {
   Level& L = H.L[g];
   const double omega = H.p.omega;
+  if (!transpose) STM_TRY(ensure_inverse_limbs(H, g, s));
   if (H.p.smoother == STM_VANKA_COLOURED) {
     for (int col = 0; col < (1 << L.dim); ++col) {
       const int nc = L.colour_off[col + 1] - L.colour_off[col];
