@@ -1,5 +1,7 @@
 """Little device memory: copies that only save time are not made where they would not fit, are given back when a required
 allocation fails, and the results stay within rounding."""
+import contextlib
+
 import numpy as np
 import pytest
 
@@ -19,13 +21,19 @@ def _hierarchy(inv, X=None):
     return h, X
 
 
-def _fill(leave):
-    """All device memory but `leave` bytes."""
+@contextlib.contextmanager
+def _only(left):
+    """Takes all device memory but `left` bytes."""
     import torch
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
-    free, _ = torch.cuda.mem_get_info()
-    return torch.empty(max(0, free - leave), dtype=torch.uint8, device="cuda")
+    hold = torch.empty(max(0, torch.cuda.mem_get_info()[0] - left), dtype=torch.uint8, device="cuda")
+    try:
+        yield
+    finally:
+        torch.cuda.synchronize()
+        del hold
+        torch.cuda.empty_cache()
 
 
 def _rows(a, b):
@@ -41,16 +49,14 @@ def test_cell_solves_without_room_and_given_back():
     r = torch.from_numpy(rng.standard_normal(n)).cuda()
     fast, slow, after, x, y = (torch.zeros_like(r) for _ in range(5))
     h.vanka_sweep(g, r, fast)  # makes the copy: 2,048 cells of 170 x 170, 473 MB
-    hold = _fill(256 << 20)
-    h2.vanka_sweep(g, r, slow)  # no room for one
-    del hold
+    with _only(256 << 20):
+        h2.vanka_sweep(g, r, slow)  # no room for one
     assert _rows(slow, fast) < 1e-12
     h2.close()
     # a Krylov basis of 61 vectors (63 MB) into 40 MB: the copy goes
-    hold = _fill(40 << 20)
-    assert h.gmres_solve(r, x, rtol=1e-9)["converged"]
-    h.vanka_sweep(g, r, after)
-    del hold
+    with _only(40 << 20):
+        assert h.gmres_solve(r, x, rtol=1e-9)["converged"]
+        h.vanka_sweep(g, r, after)
     assert _rows(after, fast) < 1e-12
     h.spmv(g, x, y)
     assert float((y - r).norm() / r.norm()) < 2e-9
@@ -66,8 +72,7 @@ def test_multi_products_without_room():
     h.close()
     # room for the vectors (0.95 GB) but not for the operands of the products (0.41 GB) as well
     h, _ = _hierarchy("bf16", X)
-    hold = _fill(1200 << 20)
-    h.gmres_solve_multi(B, slow, rtol=1e-9, restart=8, max_iter=60)
-    del hold
+    with _only(1200 << 20):
+        h.gmres_solve_multi(B, slow, rtol=1e-9, restart=8, max_iter=60)
     assert _rows(slow, fast) < 1e-7
     h.close()
