@@ -285,6 +285,7 @@ struct Hierarchy {
   // work vectors for one column and for 32 interleaved columns, the latter's partial sums
   bool coarse_slab = false;
   int cs_nx = 0, cs_t = 0, cs_maxnb = 0;
+  double cs_scale = 1.0;          // pressure_scale of the factors
   long long *cs_off = nullptr, *cs_wpos = nullptr;
   int *cs_perm = nullptr, *cs_exps = nullptr;
   void* cs_words = nullptr;
@@ -374,6 +375,9 @@ template <typename T>
 stm_status device_alloc(Hierarchy& H, T** p, size_t bytes) { return device_alloc(H, (void**)p, bytes); }
 void free_spmm_digits(Level& L);
 stm_status factor_coarse(Hierarchy& H, cudaStream_t s);
+// A power of two by which the pressure rows and columns of a level's systems are multiplied before they are inverted, so
+// that coupling and velocity blocks are of one size: digits and pivots then see neither the time step nor the mesh width.
+double pressure_scale(const Hierarchy& H, const Level& L);
 stm_status ensure_transpose(Hierarchy& H, int g, cudaStream_t s);
 // Dense FP64 products and inverses on the tensor cores (kernels_dense.cu). An operand is cut into digits in
 // a slot of the work space: as row operand (the left factor, scaled per row) or as column operand.

@@ -2,6 +2,9 @@
 // rows and columns of the ASSEMBLED global matrix on the cell's DoFs (Sec. 4.4), stored column-major per cell
 // in FP64, FP32 or BF16.
 //
+// Pressure rows and columns are inverted near the size of the velocity ones (pressure_scale): without it the residual
+// |A B - I| of an inverse against |A||B| grew with falling time steps (3D dG(0): 6e-15 at tau = 1e-2, 2e-10 at 1e-8;
+// with it 6e-15 and 2e-14).
 // One CTA per cell: blocked Gauss-Jordan elimination with partial pivoting (largest |pivot| in the column,
 // lowest row on ties), 16 pivots per panel. A panel runs in shared memory on the FP64 pipe and ends as a block
 // transform M; after the panel's row exchanges every other column c becomes (c with the panel's rows
@@ -64,6 +67,7 @@ struct CellArgs {
   const long long* rowptr;
   const double* val;
   int C, d, nv, np, nt, n, ld;
+  double scale;     // of the pressure rows and columns while the matrix is inverted
   double* scratch;  // [CTAs][n * n], or null: the matrix is kept in shared memory
   int* flag;
   long long* bad;
@@ -102,7 +106,7 @@ template <typename S, int kThreads>
 __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_cell_inverse(const __grid_constant__ CellArgs g, S* __restrict__ inv) {
   constexpr int kWarps = kThreads / 32;
   extern __shared__ __align__(16) unsigned char sm[];
-  const int n = g.n;
+  const int n = g.n, dnv = g.d * g.nv;
   const CellSmem L = cell_smem(n, g.scratch == nullptr);
   double* P = reinterpret_cast<double*>(sm);                 // [n][17]: the panel
   uint4* wm = reinterpret_cast<uint4*>(sm + L.words_m);      // [tiles][4][32]: M as row operand
@@ -135,6 +139,8 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_cell_inverse(const
           const long long pos = entry_pos(c, al, be, g.idx, g.cell_nodes, g.rank, g.cellrank, g.nn, g.ncell, g.rowptr,
                                           g.d, g.nv, g.np, g.nt, n);
           if (pos >= 0) v[k] = __ldg(g.val + pos);
+          if (al % g.nt >= dnv) v[k] *= g.scale;
+          if (be % g.nt >= dnv) v[k] *= g.scale;
         }
       }
 #pragma unroll
@@ -378,6 +384,8 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_cell_inverse(const
       for (int k = 0; k < 4; ++k) {
         const int e = e0 + k * kThreads, j = e / g.ld, i = e - j * g.ld;  // column-major store: element (i, j) at j * ld + i
         v[k] = e < n * g.ld && i < n ? A[(size_t)at[j] * n + i] : 0.0;
+        if (i % g.nt >= dnv) v[k] *= g.scale;
+        if (j % g.nt >= dnv) v[k] *= g.scale;
       }
 #pragma unroll
       for (int k = 0; k < 4; ++k)
@@ -418,7 +426,7 @@ stm_status factor_level(Hierarchy& H, int g, cudaStream_t s) {
     return STM_ERR_INVALID_ARG;
   }
   CellArgs a{L.idx, L.cell_nodes, L.nn, L.ncell, L.rank, L.cellrank, L.rowptr, L.val, L.C, L.dim, L.nv, L.np, L.nt,
-             n, lay.ld, nullptr, H.dflag, H.dbad};
+             n, lay.ld, pressure_scale(H, L), nullptr, H.dflag, H.dbad};
   // small blocks: four CTAs of four warps per SM, so that one's panel steps fill another's barriers; the
   // matrix in shared memory where that many fit, else in scratch
   const int per_sm = n <= 96 ? 4 : 2;

@@ -50,6 +50,8 @@ struct SlabView {
   const long long* wpos;  // [8][nx] block offsets in words, in tiles of 16 x 16 (-1: absent)
   const long long* epos;  // [8][nx] offsets in exps
   const int* perm;        // [n] permuted position of every row of J_1
+  long long block, dR;    // unknowns of a time node, the first pressure among them
+  double scale;           // the factors are those of J_1 with pressure rows and columns scaled
   const uint4* words;
   const int* exps;        // per block [row tiles x 16][column groups]
 };
@@ -64,6 +66,9 @@ struct Task {
   int nb = 0, nc = 0, tiles = 0, chunks = 0;
 };
 
+__device__ __forceinline__ double scaled(const SlabView& S, long long row, double v) {
+  return row % S.block >= S.dR ? v * S.scale : v;
+}
 __host__ __device__ __forceinline__ int groups_of(long long n, int g) { return (int)((n + g - 1) / g); }
 
 __device__ __forceinline__ Task make_task(const SlabView& S, int kind, int b, int c) {
@@ -233,7 +238,7 @@ __global__ void __launch_bounds__(32 * kWarps1) k_coarse_slab(SlabView S, const 
   const int base = transpose ? 4 : 0;
   const int nchain = max(max(t - 1, nx - 2 - t), 0), nback = max(t, nx - 1 - t);
   // gather into slab order
-  for (long long e = gt; e < S.n; e += nt) u[S.perm[e]] = r[e];
+  for (long long e = gt; e < S.n; e += nt) u[S.perm[e]] = scaled(S, e, r[e]);
   grid.sync();
   // z_b = Sinv_b r_b for every slab
   int first = 0;
@@ -277,7 +282,7 @@ __global__ void __launch_bounds__(32 * kWarps1) k_coarse_slab(SlabView S, const 
   }
   grid.sync();
   // back to the row order of J_1
-  for (long long e = gt; e < S.n; e += nt) d[e] = v[S.perm[e]];
+  for (long long e = gt; e < S.n; e += nt) d[e] = scaled(S, e, v[S.perm[e]]);
 }
 
 // --- 32 interleaved columns ---------------------------------------------------------------------------
@@ -385,7 +390,7 @@ __global__ void __launch_bounds__(256, 1) k_coarse_slab_multi(SlabView S, const 
   const int nchain = max(max(t - 1, nx - 2 - t), 0), nback = max(t, nx - 1 - t);
   for (long long e = gt; e < S.n * NR; e += nt) {
     const long long i = e / NR;
-    u[(long long)S.perm[i] * NR + (e - i * NR)] = R[e];
+    u[(long long)S.perm[i] * NR + (e - i * NR)] = scaled(S, i, R[e]);
   }
   grid.sync();
   auto units = [](const Task& T) { return groups_of(T.tiles, 4) * T.chunks; };
@@ -442,7 +447,7 @@ __global__ void __launch_bounds__(256, 1) k_coarse_slab_multi(SlabView S, const 
   }
   for (long long e = gt; e < S.n * NR; e += nt) {
     const long long i = e / NR;
-    Dm[e] = v[(long long)S.perm[i] * NR + (e - i * NR)];
+    Dm[e] = scaled(S, i, v[(long long)S.perm[i] * NR + (e - i * NR)]);
   }
 }
 
@@ -489,6 +494,9 @@ SlabView view_of(const Hierarchy& H) {
   S.wpos = H.cs_wpos;
   S.epos = H.cs_wpos + 8LL * H.cs_nx;
   S.perm = H.cs_perm;
+  S.block = H.L[0].block;
+  S.dR = (long long)H.L[0].dim * H.L[0].R;
+  S.scale = H.cs_scale;
   S.words = (const uint4*)H.cs_words;
   S.exps = H.cs_exps;
   return S;

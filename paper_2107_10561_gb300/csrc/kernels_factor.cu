@@ -110,26 +110,30 @@ __global__ void k_gj_colswap(double* A, long long n, int k, const int* piv) {
 // ---------------------------------------------------------------------------------------------
 
 // Dense slab blocks from the CSR of J_0: row r of slab b (permuted index pr = iperm[r]) scatters its
-// entries into D_b (same slab), Lo_b (slab b-1) or Up_b (slab b+1); anything else flags an error.
+// entries into D_b (same slab), Lo_b (slab b-1) or Up_b (slab b+1); anything else flags an error. Pressure
+// rows and columns (from dR on in every time node's block) are scaled.
 __global__ void k_slab_blocks(const long long* __restrict__ rowptr, const int* __restrict__ col,
                               const double* __restrict__ val, long long n, const int* __restrict__ iperm,
                               const int* __restrict__ blk, const long long* __restrict__ off,
                               const long long* __restrict__ dpos, const long long* __restrict__ lpos,
-                              const long long* __restrict__ upos, double* __restrict__ store, int* flag) {
+                              const long long* __restrict__ upos, double* __restrict__ store, int* flag,
+                              long long block, long long dR, double scale) {
   for (long long r = blockIdx.x; r < n; r += gridDim.x) {
+    const double fr = r % block >= dR ? scale : 1.0;
     const int pr = iperm[r];
     const int b = blk[pr];
     const long long i = pr - off[b];
     const long long nb = off[b + 1] - off[b];
     for (long long e = rowptr[r] + threadIdx.x; e < rowptr[r + 1]; e += blockDim.x) {
       const int pc = iperm[col[e]];
+      const double v = val[e] * (col[e] % block >= dR ? fr * scale : fr);
       const int bc = blk[pc];
       if (bc == b) {
-        store[dpos[b] + i * nb + (pc - off[b])] = val[e];
+        store[dpos[b] + i * nb + (pc - off[b])] = v;
       } else if (bc == b - 1) {
-        store[lpos[b] + i * (off[b] - off[b - 1]) + (pc - off[b - 1])] = val[e];
+        store[lpos[b] + i * (off[b] - off[b - 1]) + (pc - off[b - 1])] = v;
       } else if (bc == b + 1) {
-        store[upos[b] + i * (off[b + 2] - off[b + 1]) + (pc - off[b + 1])] = val[e];
+        store[upos[b] + i * (off[b + 2] - off[b + 1]) + (pc - off[b + 1])] = v;
       } else {
         atomicExch(flag, 1);
       }
@@ -163,13 +167,14 @@ __global__ void k_copy_block(const double* __restrict__ src, long long rows, lon
   }
 }
 
-// cinv[i][j] = Xp[iperm[i]][iperm[j]]
+// cinv[i][j] = Xp[iperm[i]][iperm[j]], the scaling undone
 __global__ void k_unpermute(const double* __restrict__ Xp, const int* __restrict__ iperm, long long n,
-                            double* __restrict__ out) {
+                            double* __restrict__ out, long long block, long long dR, double scale) {
   for (long long i = blockIdx.y; i < n; i += gridDim.y) {
     const double* src = Xp + (long long)iperm[i] * n;
+    const double fi = i % block >= dR ? scale : 1.0;
     for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n; j += (long long)gridDim.x * blockDim.x)
-      out[i * n + j] = src[iperm[j]];
+      out[i * n + j] = src[iperm[j]] * (j % block >= dR ? fi * scale : fi);
   }
 }
 
@@ -396,6 +401,7 @@ static stm_status factor_coarse_in(Hierarchy& H, cudaStream_t s) {
   const long long n = L.N;
   const int nx = L.cells[0];
   H.N0 = n;
+  H.cs_scale = pressure_scale(H, L);
   const bool use_slab = n >= kCoarseSlabMinDofs && nx >= 2;
   std::vector<int> iperm, blk;
   std::vector<long long> off;
@@ -456,7 +462,7 @@ static stm_status factor_coarse_in(Hierarchy& H, cudaStream_t s) {
     if (Xp) cudaMemsetAsync(Xp, 0, sizeof(double) * n * n, s);
     k_slab_blocks<<<(int)std::min<long long>(n, sm_count() * 32LL), 128, 0, s>>>(L.rowptr, L.colidx, L.val, n, d_iperm, d_blk,
                                                                           d_off, d_dpos, d_lpos, d_upos, store,
-                                                                          H.dflag + 1);
+                                                                          H.dflag + 1, L.block, (long long)L.dim * L.R, H.cs_scale);
     note_launch();
     if (use_slab) {
       st = twisted_slab_factors(H, L, off, iperm, store, dpos, lpos, upos, scal, s);
@@ -524,7 +530,7 @@ static stm_status factor_coarse_in(Hierarchy& H, cudaStream_t s) {
       break;
     }
     dim3 ug((unsigned)std::min<long long>((n + 255) / 256, 64), (unsigned)std::min<long long>(n, 65535));
-    k_unpermute<<<ug, 256, 0, s>>>(Xp, d_iperm, n, H.cinv);
+    k_unpermute<<<ug, 256, 0, s>>>(Xp, d_iperm, n, H.cinv, L.block, (long long)L.dim * L.R, H.cs_scale);
     note_launch();
     transpose_block(H.cinv, n, n, H.cinvT, s);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) {

@@ -3,6 +3,8 @@
 //  * J_g^T on the same, structurally symmetric pattern (values permuted once per assembly);
 //  * the coarse solve d = J_0^{-1} r as a dense matrix-vector product with the explicit inverse;
 //  * Gram-Schmidt building blocks of flexible GMRES (batched dots / updates, norms).
+#include <cmath>
+
 #include "internal.h"
 
 namespace stm {
@@ -91,6 +93,16 @@ __global__ void k_transpose_values(const long long* __restrict__ rowptr, const i
       valT[e] = v;
     }
   }
+}
+
+// Velocity blocks are about max(1, tau nu / h^2) times a cell's volume, coupling blocks tau / h times that. Coupling is kept
+// 2^4 below: at the same size pivots come from it early and grow (3D dG(0): residual of a cell inverse against |A||B|
+// 1.5e-13 instead of 6e-15), at 2^8 the digits lose again (2D dG(2): 4.7e-11 instead of 1.7e-12).
+double pressure_scale(const Hierarchy& H, const Level& L) {
+  double h = L.h[0];
+  for (int m = 1; m < L.dim; ++m) h = std::min(h, L.h[m]);
+  const double s = std::log2(std::max(h / H.p.tau, H.p.nu / h)) - 4;
+  return std::ldexp(1.0, (int)std::lround(std::max(-200.0, std::min(200.0, s))));
 }
 
 // What a later call can do without, only slower, and work space between two factorisations. Work that uses it may still
