@@ -77,7 +77,9 @@ typedef struct {
                             and the defect before restriction): STM_F64, or STM_F32 = FP32 copies
                             of J_g's values (kept in step with every assembly), FP32 products
                             and sums, FP64 vectors. STM_BF16 is rejected. The FGMRES products
-                            and true residuals are FP64 in every case; flexible GMRES (Sec. 3)
+                            and true residuals are FP64 in every case, or integer sums held to
+                            what an FP64 chain of the row's m terms may lose, m 2^-53 times
+                            the sum of |J| |x| in that row; flexible GMRES (Sec. 3)
                             keeps each preconditioned vector, so an inexact V-cycle only changes
                             the iteration count. The multi-RHS V-cycle keeps FP64 defects.
                             Zero-initialised structs get STM_F64.                              */
@@ -368,7 +370,7 @@ stm_status stm_profile_enable(stm_hierarchy* h, int enable);
 stm_status stm_profile_read(stm_hierarchy* h, int kernel_class, int level, double* total_ms, long long* launches,
                             double* bytes);
 /* Measured FP64 FMA throughput of the current device in TFLOP/s (8 independent FMA chains per thread,
- * best of two timed runs). The FP64 products with J are bound by this rate on GB300. Synchronous. */
+ * best of two timed runs). The products with J of 2D levels run at this rate on GB300. Synchronous. */
 stm_status stm_measure_fp64_peak(double* tflops, void* stream);
 /* Verification of the bounded waits of the pipelined kernels (the tensor-core smoother): one thread
  * waits on an mbarrier phase that nothing completes, with the same helper the pipelines use. The wait

@@ -388,7 +388,7 @@ struct DenseSlice {
   long long ld = 0;
   int rows = 0, cols = 0;
 };
-// C = [C0 +] alpha A B (m x k times k x n); trans: C^T is stored; columns [skip0, skip1) of C are left alone
+// C = [C0 +] alpha A B (m x k times k x n); trans: C^T is stored
 struct DenseProduct {
   int a = 0, b = 0;  // slots
   int m = 0, n = 0, k = 0;
@@ -397,7 +397,7 @@ struct DenseProduct {
   long long ldc0 = 0;
   double* C = nullptr;
   long long ldc = 0;
-  int trans = 0, skip0 = 0, skip1 = 0;
+  int trans = 0;
 };
 stm_status dense_reserve(DenseWork& w, int slot, long long rows, long long cols);
 stm_status dense_reserve_inverse(DenseWork& w, long long n);  // slots 0 and 1, the block, the pivots

@@ -134,7 +134,6 @@ struct GemmTask {
   double* C;                // row-major, ldc; trans: C[j * ldc + i]
   long long ldc;
   int trans;
-  int skip0, skip1;         // columns in [skip0, skip1) are not written
 };
 struct GemmTasks {
   GemmTask t[4];
@@ -248,7 +247,7 @@ __global__ void __launch_bounds__(kGemmThreads) k_digit_gemm(const __grid_consta
   for (int i = 0; i < 8; ++i) {
     const int r = m0 + wm + (lane >> 2) + ((i & 2) ? 8 : 0);
     const int c = n0 + wn + (i >> 2) * 8 + (lane & 3) * 2 + (i & 1);
-    if (r >= t.m || c >= t.n || (c >= t.skip0 && c < t.skip1)) continue;
+    if (r >= t.m || c >= t.n) continue;
     const int ea = t.ea[r], eb = t.eb[c];  // value: hi 2^(ea + eb - 36) + lo 2^(ea + eb - 68)
     double v = 0.0;
     if (ea != kExpZero && eb != kExpZero) v = t.alpha * scale_pow2(fma((double)hi[i], 4294967296.0, (double)lo[i]), ea + eb - 68);
@@ -805,8 +804,6 @@ stm_status dense_products(const DenseWork& w, const DenseProduct* pr, int count,
     t.C = p.C;
     t.ldc = p.ldc;
     t.trans = p.trans;
-    t.skip0 = p.skip0;
-    t.skip1 = p.skip1;
     g.t[used] = t;
     g.tiles[used++] = tiles;
     tiles += ((p.m + kTileM - 1) / kTileM) * ((p.n + kTileN - 1) / kTileN);

@@ -366,7 +366,7 @@ stm_status vec_scale_to(double* y, const double* x, const double* sc, int inv, l
 
 // part[v][blk] = partial sum of V[v] . w over the block's chunk; then out[v] = sum_blk part (fixed order)
 // Four dot products per block (w read once for the four); blockIdx.y walks the groups of four, side by side: in
-// short solves the FP64 sums are the time (74 clocks per warp and sum, 4 warps per sub-core), so neither the groups
+// short solves the FP64 sums are the time (64 clocks per warp and sum, 4 warps per sub-core), so neither the groups
 // nor the four warp sums of a group follow one another (warp u joins product u), and a warp sums as few as it can.
 // 14 products of 90,112 entries: 9.7 us with the groups one after the other, 8.6 side by side, 5.2 with fewer sums.
 __global__ void __launch_bounds__(256) k_dots_partial(const double* __restrict__ V, int nv, const double* __restrict__ w,

@@ -31,7 +31,7 @@ __device__ __forceinline__ double inflow_profile(int d, double y, double z, cons
   return gy * 4.0 * z * (vc.L2 - z) / (vc.L2 * vc.L2);
 }
 
-// FP64 sums are the time (74 clocks per warp and sum). The convection term c(w, w) needs K^2 (d + 1) of them per point,
+// FP64 sums are the time (64 clocks per warp and sum). The convection term c(w, w) needs K^2 (d + 1) of them per point,
 // time node and component; formed once there instead of in every row that tests it it takes a fifth of the sums (2D
 // dG(2), 16,128 cells: 366 -> 123 us per colour on average).
 __global__ void __launch_bounds__(256) k_cellvec(const int* __restrict__ cells, int ncells, int mode,

@@ -16,7 +16,8 @@
 //   - warp-transposed pressure rows: one lane per row, entry t of 32 consecutive rows contiguous.
 // Column indices are never read. In FP64, issue slots of the FP64 pipe are the limit (one FP64 warp
 // instruction every 16 cycles per SM); results equal the plain CSR product up to FP64 summation
-// order. FP64 values are kept on 2D levels only: the velocity rows of 3D levels are integers (kernels_limb_spmv.cu). In FP32 the arithmetic is cheap and the loads in flight per SM set the pace.
+// order. FP64 values are kept on 2D levels only: the velocity rows of 3D levels are integers
+// (kernels_limb_spmv.cu). In FP32 the arithmetic is cheap and the loads in flight per SM set the pace.
 #include "internal.h"
 
 namespace stm {

@@ -1,7 +1,7 @@
 // Two-limb integers of FP64 values: what the INT32 pipe multiplies in place of the FP64 pipe.
 // A value with |v| < 2^e is kept as the 58-bit integer v * 2^(58 - e) = h * 2^30 + l with a balanced low limb,
 // |h| <= 2^28 and |l| <= 2^29. The product of two such values is h h' * 2^60 + (h l' + l h') * 2^30 + l l': three
-// 32 x 32 -> 64 bit multiply-adds (4.3 clocks per warp and sub-core each, an FP64 multiply-add takes 74), and
+// 32 x 32 -> 64 bit multiply-adds (4.3 clocks per warp and sub-core each, an FP64 multiply-add takes 64), and
 // sums of them are exact. What is left out (l l') and what the limbs cut off lie about 2^-57 below the product of
 // the two scales. FP64 loses 2^-53 of every term instead, so the scales have to follow the terms: every kernel here
 // keeps a scale per class of unknowns (a velocity component or the pressure of one time node) on both sides and
