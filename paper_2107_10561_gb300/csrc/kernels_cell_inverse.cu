@@ -4,17 +4,17 @@
 //
 // Pressure rows and columns are inverted near the size of the velocity ones (pressure_scale): without it the residual
 // |A B - I| of an inverse against |A||B| grew with falling time steps (3D dG(0): 6e-15 at tau = 1e-2, 2e-10 at 1e-8;
-// with it 6e-15 and 2e-14).
+// with it 1e-15 and 4e-15).
 // One CTA per cell: blocked Gauss-Jordan elimination with partial pivoting (largest |pivot| in the column,
 // lowest row on ties), 16 pivots per panel. A panel runs in shared memory on the FP64 pipe and ends as a block
 // transform M; after the panel's row exchanges every other column c becomes (c with the panel's rows
 // cleared) + M c_panel. That product runs on the tensor cores over base-256 digits (digits.h: the rows of M
-// and the columns of c_panel scaled by powers of two, the 36 digit pairs above 2^-62), so the FP64 pipe (2
-// FMAs per clock and SM) carries 16 n^2 / 2 + n^2 / 16 x n operations instead of n^3. The matrix sits in
+// and the columns of c_panel scaled by powers of two, the 43 digit pairs above 2^-70: with the 36 above 2^-62
+// the residual of 85-row cells was 6e-15 against 1e-15 by FP64 FMAs), so the FP64 pipe (2 FMAs per clock and SM) carries 16 n^2 / 2 + n^2 / 16 x n operations instead of n^3. The matrix sits in
 // shared memory where it fits beside the operands, else in a scratch block that stays in L2.
 // Measured, 2,016 cells of 170 x 170: 25.0 -> 9.1 ms; 21,420 cells of 63 x 63: 14.7 -> 8.6 ms (a Gauss-
 // Jordan with n^3 FP64 FMAs in shared memory before). What bounds it now is instruction issue: 1.8 million
-// warp instructions per 170 x 170 cell, half of them in the update (36 MMAs, 32 to form digits and about
+// warp instructions per 170 x 170 cell, half of them in the update (43 MMAs, 32 to form digits and about
 // 200 to join the sums and add them, per 16 x 8 entries).
 #include "digits.h"
 #include "internal.h"
@@ -337,16 +337,16 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_cell_inverse(const
           const uint32_t y0[4] = {nx0.x, nx0.y, nx0.z, nx0.w}, y1[4] = {nx1.x, nx1.y, nx1.z, nx1.w};
           double cv[4] = {nc[0], nc[1], nc[2], nc[3]};
           if (ct + 1 < t1) load(ct + 1);
-          float acc[kDig][4];
+          float acc[kDig + 1][4];
 #pragma unroll
-          for (int d = 0; d < kDig; ++d)
+          for (int d = 0; d <= kDig; ++d)
 #pragma unroll
             for (int m = 0; m < 4; ++m) acc[d][m] = kSumZero;
 #pragma unroll
           for (int o = 0; o < kDig; ++o) {
             const uint32_t b0 = digit_pair(y0[o & 3], o >= 4), b1 = digit_pair(y1[o & 3], o >= 4);
 #pragma unroll
-            for (int d = 0; d + o < kDig; ++d) mma_f16(acc[d + o], a[d][0], a[d][1], a[d][2], a[d][3], b0, b1);
+            for (int d = 0; d < kDig && d + o <= kDig; ++d) mma_f16(acc[d + o], a[d][0], a[d][1], a[d][2], a[d][3], b0, b1);
           }
           const int ec0 = ec[8 * ct + 2 * q], ec1 = ec[8 * ct + 2 * q + 1];
 #pragma unroll
@@ -355,6 +355,7 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) k_cell_inverse(const
             // sums of at most 8 pairs x 16 terms x 2^14
             long long hi, lo;
             join_sums(acc, m, hi, lo);
+            lo += (__float_as_int(acc[kDig][m]) - 0x4B400000 + 128) >> 8;  // the next digit's pairs, rounded
             const int er = m < 2 ? e0 : e8, ecj = (m & 1) ? ec1 : ec0;
             if (er != kExpZero && ecj != kExpZero) cv[m] += join_pow2(hi, lo, er + ecj - 124 + 56);
             if (r < n && j < n && (j < p0 || j >= p0 + w)) A[(size_t)j * n + r] = cv[m];
