@@ -362,7 +362,7 @@ stm_status assemble_level(Hierarchy& H, int g, double nu, cudaStream_t s);
 stm_status factor_level(Hierarchy& H, int g, cudaStream_t s);
 // FP64 inverses: their copy in limbs, made before the first cell solves that gain from it where there is room, and the cell
 // solves with it (kernels_limb_vanka.cu)
-bool limb_cells_pay(int nc);
+bool limb_cells_pay(int dim, int nc);
 stm_status ensure_inverse_limbs(Hierarchy& H, int g, cudaStream_t s);
 void free_inverse_limbs(Level& L);
 stm_status vanka_limbs(const Level& L, const double* t, const int* cells, int nc, double* scatter, double omega,

@@ -3,8 +3,7 @@
 //
 // Every entry of an inverse is read once and needs one multiply-add; in FP64 that is the limit (2D dG(2), 16,384 cells,
 // 528 MB: 150 us against 78 us for the bytes at the measured copy rate). The inverses are therefore kept a second time as
-// two-limb integers (limbs.h), three integer multiply-adds each: 105 us; 2D dG(1) 97 -> 65 us, 3D dG(0) 280 -> 219,
-// 3D dG(1) (2,048 cells) 115 -> 108.
+// two-limb integers (limbs.h), three integer multiply-adds each: 105 us; 2D dG(1) 97 -> 65 us, 3D dG(0) 280 -> 219.
 //   - A sum of integers has one scale. An inverse has an exponent per row and class of columns (a velocity component or
 //     the pressures of one time node), t one per class; a class's columns are summed at the product of the two and the
 //     sum is shifted to the largest such product of the row. What is cut off is 2^-57 of that product. The classes'
@@ -16,9 +15,8 @@
 //   - A warp per cell, whole lines per load; lanes own row pairs and t's limbs are broadcast from shared memory, so
 //     a column costs a load, a shared load and six multiply-adds per lane. Exponents and the first columns are on their
 //     way while t is cut.
-//   - Fewer cells than four fifths of the resident warps (1,945) stay with the FP64 kernel, which takes several warps per
-//     cell (3D dG(1), 1,536 cells, whole sweep: 185 against 168 us; with several warps here 360 cells took 46 us against
-//     31), and so does the transpose (2D dG(2): 204 us against 145; the scales of its products differ from row to row of
+//   - Few cells stay with the FP64 kernel, which takes several warps per cell (limb_cells_pay; 3D dG(1), 1,536 cells,
+//     whole sweep: 185 against 168 us; with several warps here 360 cells took 46 us against 31), and so does the transpose (2D dG(2): 204 us against 145; the scales of its products differ from row to row of
 //     the inverse and class of columns). So do cells of fewer than 32 rows (2D dG(0): 21) and levels without
 //     room for the second copy, which is made on the first solve and given back when memory runs short.
 //   - Cells with an infinity or a NaN, in the inverse or in t, are summed in FP64 from the FP64 inverses.
@@ -272,7 +270,14 @@ stm_status launch_cells(const Level& L, const double* t, const int* cells, int n
 
 }  // namespace
 
-bool limb_cells_pay(int nc) { return 5 * nc > 4 * 8 * kCtas * sm_count(); }
+// In V-cycles, whose residuals send some rows to the FP64 sums, against the FP64 kernel. 2D, from four fifths of the
+// resident warps on (1,945 cells): dG(1), 4,096 cells 29 -> 24 us, 16,384 98 -> 66; dG(2), 2,560 34 -> 32, 4,096 43 -> 35,
+// 16,384 150 -> 107. 3D, from one and a half rounds of them on (3,648 cells): dG(0), 2,048 cells 41 -> 48 us, 3,072 70 -> 74,
+// 4,608 90 -> 76, 16,384 281 -> 214; dG(1), 2,048 116 -> 130, 3,072 168 -> 204, 4,608 243 -> 234, 16,384 854 -> 680.
+bool limb_cells_pay(int dim, int nc) {
+  const int warps = 8 * kCtas * sm_count();
+  return dim == 2 ? 5 * nc > 4 * warps : 2 * nc > 3 * warps;
+}
 
 // The elements whose cells have 32 rows and more and whose inverse is formed at all: 42 and 63 rows in 2D, 85 and 170 in 3D
 #define STM_CELLS(L, call)                          \
@@ -300,7 +305,7 @@ stm_status ensure_inverse_limbs(Hierarchy& H, int g, cudaStream_t s) {
   const int ld = inv_layout(L.n, STM_F64).ld, nk = L.K * (L.dim + 1);
   // the coloured smoother solves on the cells of one colour at a time
   const int nc = H.p.smoother == STM_VANKA_COLOURED ? L.C >> L.dim : L.C;
-  if (ld % 2 || L.n < 32 || L.n > 192 || !limb_cells_pay(nc)) return STM_OK;
+  if (ld % 2 || L.n < 32 || L.n > 192 || !limb_cells_pay(L.dim, nc)) return STM_OK;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   STM_CUDA(cudaStreamIsCapturing(s, &capture));
   if (capture != cudaStreamCaptureStatusNone) return STM_OK;

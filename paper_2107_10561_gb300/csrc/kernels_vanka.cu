@@ -418,7 +418,7 @@ static stm_status launch_local(Hierarchy& H, Level& L, int level, const double* 
   ProfScope ps(&H, STM_KCLASS_VANKA_LOCAL, s, (double)nc * ((double)L.n * L.n * storage_size(prec) + 20.0 * L.n),
                level);
   const double omega = H.p.omega;
-  if (prec == STM_F64 && L.lim_current && !transpose && limb_cells_pay(nc)) return vanka_limbs(L, t, cells, nc, scatter, omega, s);
+  if (prec == STM_F64 && L.lim_current && !transpose && limb_cells_pay(L.dim, nc)) return vanka_limbs(L, t, cells, nc, scatter, omega, s);
   if (!transpose) {
     const VGeom g = vanka_geometry(L.n, lay, prec);
     if (prec == STM_F64) launch_fwd<double>(L, L.inv, lay.vb, g, t, cells, nc, scatter, omega, s);

@@ -7,7 +7,8 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 CASES = [(2, 1, 2, (3, 2)), (2, 1, 5, (16, 4)), (2, 2, 2, (5, 3)), (2, 2, 4, (10, 4)), (3, 0, 2, (3, 2, 2)),
-         (3, 0, 2, (16, 4, 4)), (3, 1, 2, (2, 3, 2)), (3, 1, 2, (16, 4, 4))]
+         (3, 0, 2, (16, 4, 4)), (3, 1, 2, (2, 3, 2)), (3, 1, 2, (16, 4, 4)),
+         (3, 0, 2, (16, 6, 5)), (3, 1, 2, (16, 6, 5))]
 
 
 def _vectors(rng, n, k, dim, R):
