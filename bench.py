@@ -358,7 +358,7 @@ def spmm_roofline(f, nnz, kern, workload_name):
     """The multi-RHS SpMM Y = J_g X (32 columns) in FP64 accuracy, finest level, against the copy bandwidth.
 
     On the workload it is quoted for the product runs on the tensor cores over base-256 digits and is bound by
-    instruction issue (forming digits). achieved = algorithmic bytes (J once, X and Y once) per launch / average
+    chains of dependent instructions (forming digits, joining sums). achieved = algorithmic bytes (J once, X and Y once) per launch / average
     event time per launch; peak = measured copy bandwidth; fp64_tflops_equivalent = 2 * nnz * 32 FLOP over the
     same time; share = the finest-level SpMM event time over the event time of all classes in the profiled solve."""
     if f["ms"] <= 0 or f["launches"] == 0:
@@ -369,7 +369,7 @@ def spmm_roofline(f, nnz, kern, workload_name):
     gbs = f["bytes"] / (f["ms"] * 1e-3) / 1e9
     total = sum(v["ms"] for v in kern.values())
     traffic = recorded_traffic(workload_name, "k_spmm_digits")
-    return {"kernel": "k_spmm_digits (Y = J_g X, 32 columns, finest level)", "bound": "issue",
+    return {"kernel": "k_spmm_digits (Y = J_g X, 32 columns, finest level)", "bound": "latency",
             "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
             "traffic": traffic["per_launch_bytes"] if traffic else None,
             "traffic_source": traffic["source"] if traffic else "no capture of the current kernel source",

@@ -11,11 +11,12 @@
 // cleared) + M c_panel. That product runs on the tensor cores over base-256 digits (digits.h: the rows of M
 // and the columns of c_panel scaled by powers of two, the 43 digit pairs above 2^-70: with the 36 above 2^-62
 // the residual of 85-row cells was 6e-15 against 1e-15 by FP64 FMAs), so the FP64 pipe (2 FMAs per clock and SM) carries 16 n^2 / 2 + n^2 / 16 x n operations instead of n^3. The matrix sits in
-// shared memory where it fits beside the operands, else in a scratch block that stays in L2.
-// Measured, 2,016 cells of 170 x 170: 25.0 -> 9.1 ms; 21,420 cells of 63 x 63: 14.7 -> 8.6 ms (a Gauss-
-// Jordan with n^3 FP64 FMAs in shared memory before). What bounds it now is instruction issue: 1.8 million
-// warp instructions per 170 x 170 cell, half of them in the update (43 MMAs, 32 to form digits and about
-// 200 to join the sums and add them, per 16 x 8 entries).
+// shared memory where it fits beside the operands, else in a scratch block that L2 holds for the most part.
+// Measured, 2,016 cells of 170 x 170: 25.0 -> 9.6 ms; 21,420 cells of 63 x 63: 14.7 -> 9.3 ms (a Gauss-
+// Jordan with n^3 FP64 FMAs in shared memory before). What bounds it now are chains of dependent instructions
+// at 16 warps per SM (issue slots 46 % used, FP64 pipe 42 %): 2.5 million warp instructions per 170 x 170 cell,
+// half of them in the update (43 MMAs, 32 to form digits and about 200 to join the sums and add them, per 16 x 8
+// entries).
 #include "digits.h"
 #include "internal.h"
 
